@@ -1569,9 +1569,13 @@ VL_API vl_status vl_result_masks(const vl_result* r, uint32_t* dst, int32_t dst_
   DeviceGuard dg(r->ctx->device);
   const size_t words = (size_t)r->H * r->Wp;
   cudaError_t e = wait_result(r, S(stream));
-  for (int q = 0; q < r->n_roots && !e; ++q)
-    e = cudaMemcpyAsync(dst + words * q, r->roots[q], words * 4,
+  // one copy per run of roots that lie back to back (distinct roots all do):
+  // a copy each took 4 us a root, longer than a small mask takes to compute
+  for (int q = 0, end; q < r->n_roots && !e; q = end) {
+    for (end = q + 1; end < r->n_roots && r->roots[end] == r->roots[end - 1] + words;) ++end;
+    e = cudaMemcpyAsync(dst + words * q, r->roots[q], words * 4 * (size_t)(end - q),
                         dst_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, S(stream));
+  }
   if (!e && !dst_on_device) e = cudaStreamSynchronize(S(stream));
   if (e) return cuda_err(r->ctx, e, "copying result masks");
   return VL_OK;
