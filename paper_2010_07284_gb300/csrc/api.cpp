@@ -206,7 +206,7 @@ vl_status batch_build(vl_context* ctx, const vl_job* jobs, int n_jobs, cudaStrea
     int H, W, Wp, pitch;
     int gty, gtx, cty, ctx_, ctiles, cth;
     std::vector<int> need;
-    size_t off_images, off_slotptrs, off_pct, off_slots, off_rz, set_bytes, set_off[3];
+    size_t off_images, off_slotptrs, off_pct, off_slots, off_rz, set_bytes, set_off[2];
     size_t off_roots, off_status, off_planes, off_num;
     int n_table;  // image table: the formula's images, then its number images
     int step_base;
@@ -383,13 +383,12 @@ vl_status batch_build(vl_context* ctx, const vl_job* jobs, int n_jobs, cudaStrea
     I.off_num = take(sizeof(float) * (size_t)I.H * I.pitch * P.n_num_images);
     I.off_slots = take(mask_bytes * P.n_inter_slots);
     const size_t tstate = (size_t)I.ctiles * ccl_tile_cap_host(I.Wp, I.cth);
-    // select scratch sets: G (2 * P_px keys), tpar, tflag, each 256-byte aligned
+    // select scratch sets: G (2 * P_px keys) and the tiles' state, 256-byte aligned
     {
       size_t o = 0;
       auto sub = [&](size_t bytes) { o = align_up(o, 256); size_t r = o; o += bytes; return r; };
       I.set_off[0] = sub(2 * P_px * 4);
       I.set_off[1] = sub(tstate * 4);
-      I.set_off[2] = sub(tstate);
       I.set_bytes = align_up(o, 256);
       I.off_rz = take(I.set_bytes * (size_t)P.n_scratch_sets);
     }
@@ -483,8 +482,7 @@ vl_status batch_build(vl_context* ctx, const vl_job* jobs, int n_jobs, cudaStrea
     d.planes = reinterpret_cast<uint32_t*>(tb + I.off_planes);
     d.rzs = reinterpret_cast<unsigned char*>(tb + I.off_rz);
     d.set_bytes = (int64_t)I.set_bytes;
-    d.off_tpar = (int64_t)I.set_off[1];
-    d.off_tflag = (int64_t)I.set_off[2];
+    d.off_state = (int64_t)I.set_off[1];
     d.tile_cap = ccl_tile_cap_host(I.Wp, I.cth);
     d.c_th = I.cth;
     d.status = status_dev + j;
@@ -824,14 +822,13 @@ vl_status plain_enqueue(vl_context* ctx, const Plan& P, vl_image* const* imgs, i
     const int tcap = ccl_tile_cap_host(Wp, ccl_rows(g));
     size_t off = 0;
     auto take = [&](size_t b) { off = align_up(off, 256); size_t o = off; off += b; return o; };
-    const size_t oG = take(2 * px * 4), oP = take(tiles * tcap * 4), oT = take(tiles * tcap);
+    const size_t oG = take(2 * px * 4), oP = take(tiles * tcap * 4);
     if ((e = dev_alloc(ctx, align_up(off, 256), st, &scratch)))
       return cuda_err(ctx, e, "allocating select scratch");
     char* p = static_cast<char*>(scratch->ptr);
     sc.G = reinterpret_cast<int32_t*>(p + oG);
     sc.tile_cap = tcap;
     sc.tpar = reinterpret_cast<int32_t*>(p + oP);
-    sc.tflag = reinterpret_cast<uint8_t*>(p + oT);
   }
   const int N = (int)P.exec.size();
   std::vector<int> uses(N, 0), root_slot(N, -1);
@@ -978,7 +975,7 @@ VL_API vl_status vl_context_create(const vl_config* cfg, vl_context** out) {
   c->gtww = c->cfg.tile_words > 0 ? c->cfg.tile_words : 32;
   c->hmax = 8;
   const int bh = c->gth + 2 * c->hmax, bw = c->gtww + 2;
-  const size_t budget = std::max<size_t>(ccl_smem_bytes(), 64 * 1024);
+  const size_t budget = kGroupBudget;
   c->nb = (int)std::min<size_t>(64, budget / ((size_t)bh * bw * 4));
   if (c->nb < 4) { delete c; return VL_ERR_ARG; }
   c->pp.group_buffers = c->nb;
@@ -1260,7 +1257,7 @@ static PlanParams default_plan_params() {
   PlanParams pp;
   pp.hmax = 8;
   const int bh = 32 + 2 * pp.hmax, bw = 32 + 2;
-  const size_t budget = std::max<size_t>(ccl_smem_bytes(), 64 * 1024);
+  const size_t budget = kGroupBudget;
   pp.group_buffers = (int)std::min<size_t>(64, budget / ((size_t)bh * bw * 4));
   return pp;
 }

@@ -26,17 +26,41 @@ namespace vl {
 
 constexpr uint32_t FULL = 0xFFFFFFFFu;
 
+// Pairs the first links of a tile may leave over (more are united at once).
+constexpr int CCL_PEND = 4096;
+static_assert(CCL_MAXRUNS <= 16384, "runs are packed into 16 bits with two flags");
+
 struct CclSmem {
   uint32_t m[CCL_TH][CCL_TWW];   // rows of the tile
   uint32_t u[CCL_NS][CCL_TWW];   // strip unions (row 2k | row 2k+1)
   uint32_t st[CCL_NS][CCL_TWW];  // strip-run starts
+  uint32_t sd[CCL_NS][CCL_TWW];  // first seed column of every strip run, per word
   int32_t pre[CCL_NS][CCL_TWW];  // starts before each word, per strip
   int32_t qc[CCL_NS][CCL_TWW];   // boundary anchor entering each word
+  int32_t cnt[CCL_NS];           // runs of each strip
   int32_t base[CCL_NS + 1];      // first strip-run id of each strip
-  int32_t nruns;
-  int32_t pad;
+  int32_t npend;                 // pairs offered to pend (may exceed its size)
+  int32_t nlist;                 // border roots listed
+  uint32_t pend[CCL_PEND];       // unions left over by the first links: run << 16 | run;
+                                 //   later the list of border roots
   int32_t parent[CCL_MAXRUNS];   // union-find; after labelling a root holds -(value + 2)
-  uint8_t flag[CCL_MAXRUNS];     // bit0 seed, bit1 on tile border, bit2 selected
+  uint8_t flag[CCL_MAXRUNS];     // of roots: bit0 seed, bit1 on tile border
+};
+
+// What the select pass of rho keeps of a tile: its rows and strips, and a
+// 16-bit code per strip run (the run's root, or for a root RZ_ROOT with
+// RZ_SEED when it holds a seed pixel and RZ_SEL when it is selected).
+constexpr uint32_t RZ_ROOT = 0x8000u, RZ_SEED = 0x4000u, RZ_SEL = 0x2000u;
+struct RzSmem {
+  uint32_t m[CCL_TH][CCL_TWW];
+  uint32_t u[CCL_NS][CCL_TWW];
+  uint32_t st[CCL_NS][CCL_TWW];
+  uint32_t sd[CCL_NS][CCL_TWW];  // (unused)
+  int32_t pre[CCL_NS][CCL_TWW];
+  int32_t cnt[CCL_NS];
+  int32_t base[CCL_NS + 1];
+  uint32_t list[CCL_MAXBORDER];  // border roots: run | RZ_SEL << 16 when selected
+  uint16_t code[CCL_MAXRUNS];
 };
 
 struct CclGeom {
@@ -276,7 +300,8 @@ VL_DEV uint32_t strip_starts(uint32_t a, uint32_t b, uint32_t al, uint32_t bl, i
 }
 
 // Strip run holding tile pixel x of strip k (x must be set in the strip).
-VL_DEV int sid(const CclSmem& s, int k, int x) {
+template <class Smem>
+VL_DEV int sid(const Smem& s, int k, int x) {
   const int w = x >> 5;
   return s.base[k] + s.pre[k][w] + __popc(s.st[k][w] & le_mask(x & 31)) - 1;
 }
@@ -285,130 +310,144 @@ VL_DEV bool mbit(const CclSmem& s, int row, int x) {
   return (s.m[row][x >> 5] >> (x & 31)) & 1u;
 }
 
-// Dilation of mask `a` at (image row y, image word w) for one warp whose
-// lanes hold consecutive words w0 + lane; lanes >= n are idle but take part
-// in the shuffles.  Pixels outside the image are false.
-VL_DEV uint32_t warp_near_row(const uint32_t* a, int H, int W, int Wp, int y,
-                              int w0, int lane, int n, int conn) {
-  int w = w0 + lane;
-  bool in = lane < n;
-  uint32_t u = 0, c = 0, d = 0;
-  if (in) {
-    if (y > 0) u = ldcg(&a[(size_t)(y - 1) * Wp + w]);
-    c = ldcg(&a[(size_t)y * Wp + w]);
-    if (y + 1 < H) d = ldcg(&a[(size_t)(y + 1) * Wp + w]);
-  }
-  uint32_t ul = __shfl_up_sync(FULL, u, 1), cl = __shfl_up_sync(FULL, c, 1),
-           dl = __shfl_up_sync(FULL, d, 1);
-  uint32_t ur = __shfl_down_sync(FULL, u, 1), cr = __shfl_down_sync(FULL, c, 1),
-           dr = __shfl_down_sync(FULL, d, 1);
-  if (in && lane == 0) {
-    ul = cl = dl = 0;
-    if (w > 0) {
-      if (y > 0) ul = ldcg(&a[(size_t)(y - 1) * Wp + w - 1]);
-      cl = ldcg(&a[(size_t)y * Wp + w - 1]);
-      if (y + 1 < H) dl = ldcg(&a[(size_t)(y + 1) * Wp + w - 1]);
-    }
-  }
-  if (in && lane == n - 1) {
-    ur = cr = dr = 0;
-    if (w + 1 < Wp) {
-      if (y > 0) ur = ldcg(&a[(size_t)(y - 1) * Wp + w + 1]);
-      cr = ldcg(&a[(size_t)y * Wp + w + 1]);
-      if (y + 1 < H) dr = ldcg(&a[(size_t)(y + 1) * Wp + w + 1]);
-    }
-  }
-  if (!in) return 0;
-  return near_word(ul, u, ur, cl, c, cr, dl, d, dr, conn) & vmask(w, W);
-}
-
-// Anchor of the boundary run starting at tile pixel x of boundary b: the
-// strip run of its first pixel (upper strip if the upper row is set there).
-VL_DEV int anchor_at(const CclSmem& s, int b, int x) {
-  return mbit(s, 2 * b + 1, x) ? sid(s, b, x) : sid(s, b + 1, x);
-}
-
 // Root of strip run i once roots are encoded (parent[root] < 0).
 VL_DEV int root_of(const CclSmem& s, int i) {
   const int p = s.parent[i];
   return p >= 0 ? p : i;
 }
 
-// Label one tile in shared memory.  Returns false (uniformly, after a block
-// barrier) if the tile has more strip runs than the shared arrays hold, which
-// cannot happen for CCL_TH x CCL_TWW tiles; the caller then skips the tile.
-// On success: s.parent[i] of a non-root is its root (smallest id); a root
-// holds a negative value, with `min_pixel` -(component's minimum linear pixel
-// index + 2); s.flag[root] has bit0 when a seed pixel lies in the component
-// (seed = mask and N phi1, if phi1 is given) and bit1 when the component
-// reaches the tile border.  Must be called by every thread of the block.
-// Rows of the tile into shared memory, strip unions, strip-run starts and
-// their prefix counts.  Returns the number of strip runs (uniform, after a
-// block barrier).
-VL_DEV int ccl_tile_strips(CclSmem& s, const uint32_t* mask, const CclGeom& g, int conn) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int nw = blockDim.x >> 5;
+// The two rows of the warp's strip (a warp takes one: a tile has no more
+// strips than the block has warps), loaded ahead of ccl_tile_strips.
+static_assert(EXEC_WARPS >= CCL_NS, "a warp per strip");
+struct StripRows { uint32_t a, b; };
+VL_DEV StripRows ccl_load_rows(const uint32_t* mask, const CclGeom& g) {
+  const int lane = threadIdx.x & 31, r0 = 2 * (threadIdx.x >> 5);
+  StripRows q{0u, 0u};
+  if (lane < g.tww && r0 < g.th) {
+    const size_t at = (size_t)(g.r0 + r0) * g.Wp + g.w0 + lane;
+    q.a = ldcg(&mask[at]);
+    if (r0 + 1 < g.th) q.b = ldcg(&mask[at + g.Wp]);
+  }
+  return q;
+}
+
+// Rows of the tile into shared memory, strip unions, strip-run starts, their
+// counts before each word and per strip, and, with phi1, the seed columns:
+// all loads of a strip are in flight together.  Every warp then adds the
+// strips' counts up for itself: lane l returns the number of strip runs
+// before strip l (lane 31: all of them), the same in every warp.  s.base is
+// written by warp 0: a block barrier before it is read.
+template <class Smem>
+VL_DEV int ccl_tile_strips(Smem& s, StripRows rows, const uint32_t* phi1, const CclGeom& g, int conn) {
+  const int lane = threadIdx.x & 31, k = threadIdx.x >> 5;
   const int ns = (g.th + 1) >> 1;
-  // 1. rows, strip unions, strip-run starts, per-strip prefix counts
-  for (int k = warp; k < ns; k += nw) {
-    const int r0 = 2 * k, r1 = 2 * k + 1;
-    uint32_t a = 0, b = 0;
-    if (lane < g.tww) {
-      // padding bits (columns >= W) are cleared here, so that no later pass
-      // can see a pixel outside the image whatever the caller's buffer holds
-      const uint32_t vm = vmask(g.w0 + lane, g.W);
-      a = ldcg(&mask[(size_t)(g.r0 + r0) * g.Wp + g.w0 + lane]) & vm;
-      if (r1 < g.th) b = ldcg(&mask[(size_t)(g.r0 + r1) * g.Wp + g.w0 + lane]) & vm;
+  if (k < ns) {
+    const int y = g.r0 + 2 * k, w = g.w0 + lane;
+    const bool in = lane < g.tww;
+    uint32_t f[4] = {0u, 0u, 0u, 0u}, e[4] = {0u, 0u, 0u, 0u};
+    if (phi1 != nullptr) {
+      // phi1 around the strip, rows y - 1 .. y + 2 of the image, and beside
+      // the tile, left of lane 0 and right of the last lane (a tile has at
+      // least four words: they are two lanes)
+      const int we = lane == 0 ? w - 1 : w + 1;
+      const bool edge = in && (lane == 0 || lane == g.tww - 1) && we >= 0 && we < g.Wp;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int yy = y - 1 + q;
+        const bool row = yy >= 0 && yy < g.H;
+        if (row && in) f[q] = ldcg(&phi1[(size_t)yy * g.Wp + w]);
+        if (row && edge) e[q] = ldcg(&phi1[(size_t)yy * g.Wp + we]);
+      }
     }
+    // padding bits (columns >= W) are cleared here, so that no later pass
+    // can see a pixel outside the image whatever the caller's buffer holds
+    const uint32_t vm = in ? vmask(w, g.W) : 0u, a = rows.a & vm, b = rows.b & vm;
     uint32_t al = __shfl_up_sync(FULL, a, 1), bl = __shfl_up_sync(FULL, b, 1);
     if (lane == 0) al = bl = 0;
     const uint32_t st = strip_starts(a, b, al, bl, conn);
     const int c = __popc(st);
     const int incl = warp_incl_scan(c, lane);
-    s.m[r0][lane] = a;
-    s.m[r1][lane] = b;
+    s.m[2 * k][lane] = a;
+    s.m[2 * k + 1][lane] = b;
     s.u[k][lane] = a | b;
     s.st[k][lane] = st;
     s.pre[k][lane] = incl - c;
-    if (lane == 31) s.base[k + 1] = incl;
+    if (lane == 31) s.cnt[k] = incl;
+    if (phi1 != nullptr) {
+      // N phi1 on the two rows: vertical first, then the neighbour words
+      uint32_t c0, c1, v0 = 0, v1 = 0, e0, e1;
+      if (conn == 8) {
+        c0 = f[0] | f[1] | f[2];
+        c1 = f[1] | f[2] | f[3];
+        e0 = e[0] | e[1] | e[2];
+        e1 = e[1] | e[2] | e[3];
+      } else {
+        c0 = f[1];
+        c1 = f[2];
+        v0 = f[0] | f[2];
+        v1 = f[1] | f[3];
+        e0 = e[1];
+        e1 = e[2];
+      }
+      uint32_t l0 = __shfl_up_sync(FULL, c0, 1), l1 = __shfl_up_sync(FULL, c1, 1);
+      uint32_t q0 = __shfl_down_sync(FULL, c0, 1), q1 = __shfl_down_sync(FULL, c1, 1);
+      if (lane == 0) { l0 = e0; l1 = e1; }
+      if (lane == g.tww - 1) { q0 = e0; q1 = e1; }
+      const uint32_t z = (a & (v0 | hdil(l0, c0, q0))) | (b & (v1 | hdil(l1, c1, q1)));
+      s.sd[k][lane] = first_in_segments(z, st);
+    }
   }
   __syncthreads();
-  if (warp == 0) {
-    const int v = (lane < ns) ? s.base[lane + 1] : 0;
-    const int incl = warp_incl_scan(v, lane);
-    __syncwarp();
+  const int v = lane < ns ? s.cnt[lane] : 0;
+  const int incl = warp_incl_scan(v, lane);
+  if (k == 0) {
     if (lane < ns) s.base[lane] = incl - v;
-    if (lane == 31) s.nruns = incl;
     if (lane == 31) s.base[ns] = incl;
   }
-  __syncthreads();
-  return s.nruns;
+  return lane == 31 ? incl : incl - v;
 }
 
-VL_DEV bool ccl_tile_label(CclSmem& s, const uint32_t* mask, const uint32_t* phi1,
-                           const CclGeom& g, int conn, bool min_pixel, int32_t* status) {
+// Label one tile in shared memory.  Returns the number of strip runs, or -1
+// (uniformly) if the tile has more than the shared arrays hold, which cannot
+// happen for CCL_TH x CCL_TWW tiles; the caller then skips the tile.  On
+// success: s.parent[i] of a non-root is its root (smallest id); a root holds
+// a negative value -(v + 2).  With phi1 (the select of rho), v is a border
+// pixel of the component (INT_MIN: it has none) and s.flag[root] bit0 says
+// whether it holds a seed pixel (mask and N phi1); without (labels), v is
+// the component's minimum linear pixel index.  s.pend[0 .. s.nlist) lists
+// the roots of the components that reach the tile border.  Must be called by
+// every thread of the block; a block barrier at the end.
+VL_DEV int ccl_tile_label(CclSmem& s, const uint32_t* mask, const uint32_t* phi1,
+                          const CclGeom& g, int conn, int32_t* status) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int nw = blockDim.x >> 5;
   const int ns = (g.th + 1) >> 1;
-  ccl_tile_strips(s, mask, g, conn);
-  const int nruns = s.nruns;
-  if (nruns > CCL_MAXRUNS) {  // uniform: every thread reads the same count
+  const int before = ccl_tile_strips(s, ccl_load_rows(mask, g), phi1, g, conn);
+  const int nruns = __shfl_sync(FULL, before, 31);
+  if (nruns > CCL_MAXRUNS) {  // uniform: every warp has the same count
     set_status(status, ST_INTERNAL | RS_TRUNS);
-    return false;
+    return -1;
   }
   for (int i = tid; i < nruns; i += blockDim.x) {
     s.parent[i] = i;
     s.flag[i] = 0;
   }
-  // 2. anchor of the boundary run entering each word from the left
+  if (tid == 0) s.npend = s.nlist = 0;
+  // 2. anchor of the boundary run entering each word from the left: the strip
+  // run of its first pixel (in the upper strip if the upper row is set there)
   for (int b = warp; b < ns - 1; b += nw) {
+    const int base_b = __shfl_sync(FULL, before, b), base_c = base_b + s.cnt[b];
     uint32_t A = 0, B = 0;
     if (lane < g.tww) { A = s.m[2 * b + 1][lane]; B = s.m[2 * b + 2][lane]; }
     uint32_t Al = __shfl_up_sync(FULL, A, 1), Bl = __shfl_up_sync(FULL, B, 1);
     if (lane == 0) Al = Bl = 0;
     const uint32_t qs = strip_starts(A, B, Al, Bl, conn);
     int last = -1;
-    if (qs) last = anchor_at(s, b, 32 * lane + 31 - __clz(qs));
+    if (qs) {
+      const int p = 31 - __clz(qs);
+      last = (A >> p) & 1u ? base_b + s.pre[b][lane] + __popc(s.st[b][lane] & le_mask(p)) - 1
+                           : base_c + s.pre[b + 1][lane] + __popc(s.st[b + 1][lane] & le_mask(p)) - 1;
+    }
     int idx = last >= 0 ? lane : -1;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -421,31 +460,28 @@ VL_DEV bool ccl_tile_label(CclSmem& s, const uint32_t* mask, const uint32_t* phi
     s.qc[b][lane] = prev < 0 ? -1 : carried;
   }
   __syncthreads();
-  // 3. unite across strip boundaries, one tree level at a time (boundary b
-  // belongs to level = trailing ones of b), so each level unites disjoint
-  // groups of strips.  Every thread takes a share of the row-run starts
-  // ("events") of one boundary word; the word's strip data sits in
-  // registers.  In each round every thread with an event links its pair of
-  // roots (atomicMin of the larger root's parent); a link that finds the
-  // larger root already linked elsewhere leaves the follow-up union (old
-  // parent, lo) to the same thread.
+  // 3. unite across the strip boundaries, all of them at once.  Every thread
+  // takes a share of the columns of one boundary word; the word's strip data
+  // sits in registers.  A row-run start ("event") links the larger of its
+  // run and the boundary run's anchor under the smaller without looking for
+  // roots: most runs (more than half of the events on noise) are linked
+  // upwards for the first time and are done with that one atomicMin.  An
+  // event whose run already had another parent leaves the pair (old parent,
+  // smaller run) in a list, so that the parents and the list together always
+  // hold the whole relation.
   const int cap = nruns + 64;
   bool ok = true;
-  for (int level = 0; (1 << level) < ns; ++level) {
-    const int step = 2 << level, first = (1 << level) - 1;  // b = first + j * step
-    const int nb = (ns - 1 - first + step - 1) / step;
-    const int pairs = nb > 0 ? nb * g.tww : 0;
+  {
+    const int pairs = (ns - 1) * g.tww;
     int T = 1;
-    while (pairs > 0 && T * 2 * pairs <= (int)blockDim.x) T *= 2;
-    const int pair = tid / T, sub = tid - (tid / T) * T;
-    const bool act = pair < pairs;
-    uint32_t A = 0, B = 0, qs = 0, evA = 0, evB = 0, stb = 0, stc = 0;
-    int b = 0, w = 0, bb = 0, bc = 0, carry = -1;
-    if (act) {
-      b = first + (pair / g.tww) * step;
-      w = pair - (pair / g.tww) * g.tww;
+    while (pairs > 0 && T < 32 && T * 2 * pairs <= (int)blockDim.x) T *= 2;
+    const int pair = tid / T, sub = tid - pair * T;
+    uint32_t A = 0, qs = 0, evA = 0, evB = 0, stb = 0, stc = 0;
+    int bb = 0, bc = 0, carry = -1;
+    if (pair < pairs) {
+      const int b = pair / g.tww, w = pair - b * g.tww;
       A = s.m[2 * b + 1][w];
-      B = s.m[2 * b + 2][w];
+      const uint32_t B = s.m[2 * b + 2][w];
       const uint32_t Al = w > 0 ? s.m[2 * b + 1][w - 1] : 0u;
       const uint32_t Bl = w > 0 ? s.m[2 * b + 2][w - 1] : 0u;
       qs = strip_starts(A, B, Al, Bl, conn);
@@ -458,132 +494,158 @@ VL_DEV bool ccl_tile_label(CclSmem& s, const uint32_t* mask, const uint32_t* phi
       // when a boundary-run or strip-run start separates it from the
       // previous one, i.e. the first row-run start of every segment that
       // begins at such a start (or at the word's left edge)
-      const uint32_t ra_ = A & ~((A << 1) | (Al >> 31));
-      const uint32_t rb_ = B & ~((B << 1) | (Bl >> 31));
-      evA = first_in_segments(ra_, qs | stb);
-      evB = first_in_segments(rb_, qs | stc);
+      const uint32_t share = T == 1 ? FULL : (((1u << (32 / T)) - 1u) << (sub * (32 / T)));
+      evA = first_in_segments(A & ~((A << 1) | (Al >> 31)), qs | stb) & share;
+      evB = first_in_segments(B & ~((B << 1) | (Bl >> 31)), qs | stc) & share;
     }
-    const int nA = __popc(evA), nE = nA + __popc(evB);
-    // this thread's events: a contiguous share [j, e1) of the pair's list
-    // (the A events, then the B events), walked by clearing lowest bits
-    const int per = (nE + T - 1) / T;
-    int j = min(nE, sub * per);
-    const int e1 = min(nE, j + per);
-    uint32_t curA = 0, curB = 0;
-    if (j < e1) {
-      if (j < nA) {
-        curA = j ? evA & ~((1u << __fns(evA, 0, j + 1)) - 1u) : evA;
-        curB = evB;
-      } else {
-        curB = j > nA ? evB & ~((1u << __fns(evB, 0, j - nA + 1)) - 1u) : evB;
+    // links u and v; true when that left the pair (old, lo)
+    auto link = [&](int u, int v, int& old, int& lo) {
+      if (u == v) return false;
+      const int hi = max(u, v);
+      lo = min(u, v);
+      old = atomicMin(&s.parent[hi], lo);
+      return old != hi && old != lo;
+    };
+    auto push = [&](bool left, int old, int lo) {
+      const unsigned lm = __ballot_sync(FULL, left);
+      if (!lm) return;
+      int at = 0;
+      if (lane == 0) at = atomicAdd(&s.npend, __popc(lm));
+      at = __shfl_sync(FULL, at, 0) + __popc(lm & ((1u << lane) - 1u));
+      if (left) {
+        if (at < CCL_PEND) s.pend[at] = ((uint32_t)old << 16) | (uint32_t)lo;
+        else ok = s_union(s.parent, old, lo, cap) && ok;  // (the list is full)
       }
-    }
-    int pu = -1, pv = -1;
-    for (int round = 0; round < 4 * CCL_MAXRUNS; ++round) {
-      const bool has = act && (pu >= 0 || j < e1);
-      if (!__any_sync(FULL, has)) break;
-      int ra = 0, rb = 0;
-      const bool from_event = has && pu < 0;
-      if (has) {
-        int u = pu, v = pv;
-        if (from_event) {
-          const bool isA = curA != 0;
-          const uint32_t cur = isA ? curA : curB;
-          const int p = __ffs(cur) - 1;
-          if (isA) curA &= curA - 1u;
-          else curB &= curB - 1u;
-          u = isA ? bb + __popc(stb & le_mask(p)) : bc + __popc(stc & le_mask(p));
-          const uint32_t qq = qs & le_mask(p);
-          if (qq) {
-            const int q = 31 - __clz(qq);
-            v = ((A >> q) & 1u) ? bb + __popc(stb & le_mask(q)) : bc + __popc(stc & le_mask(q));
-          } else {
-            v = carry >= 0 ? carry : u;
-          }
+    };
+    for (int round = 0; round < 32; ++round) {  // (at most 32 columns a word)
+      const uint32_t ev = evA | evB;
+      if (!__any_sync(FULL, ev != 0)) break;
+      bool left1 = false, left2 = false;
+      int old1 = 0, lo1 = 0, old2 = 0, lo2 = 0;
+      if (ev) {
+        const uint32_t bit = ev & (0u - ev), le = bit | (bit - 1u);
+        const int ub = bb + __popc(stb & le), uc = bc + __popc(stc & le);
+        const uint32_t qq = qs & le;
+        int v = carry;
+        if (qq) {
+          const int q = 31 - __clz(qq);
+          v = (A >> q) & 1u ? bb + __popc(stb & le_mask(q)) : bc + __popc(stc & le_mask(q));
         }
-        // both roots at once; walks that meet need no link
-        ra = u; rb = v;
-        if (!s_find2(s.parent, ra, rb, cap)) { ok = false; ra = rb = 0; }
+        if (v >= 0) {
+          if (evA & bit) left1 = link(ub, v, old1, lo1);
+          if (evB & bit) left2 = link(uc, v, old2, lo2);
+        }
+        evA &= ~bit;
+        evB &= ~bit;
       }
-      // link the larger root under the smaller; when hi was no longer a
-      // root its old parent (unless already lo) still has to meet lo
-      const bool need = has && ra != rb;
-      const int hi = max(ra, rb), lo = min(ra, rb);
-      int old = hi;
-      if (need) old = atomicMin(&s.parent[hi], lo);
-      if (has) {
-        if (from_event) ++j;
-        else pu = pv = -1;
-        if (need && old != hi && old != lo) { pu = old; pv = lo; }
+      push(left1, old1, lo1);
+      push(left2, old2, lo2);
+    }
+  }
+  __syncthreads();
+  // the listed pairs, dealt out evenly: both roots at once (walks that meet
+  // need no link), the larger linked under the smaller; a link that finds
+  // the larger root already linked elsewhere leaves the follow-up union
+  // (old parent, smaller root) to the same thread
+  {
+    const int n = min(s.npend, CCL_PEND);
+    int next = tid, pu = -1, pv = -1;
+    for (int round = 0; round < 4 * CCL_MAXRUNS; ++round) {
+      if (pu < 0 && next < n) {
+        const uint32_t e = s.pend[next];
+        pu = (int)(e >> 16);
+        pv = (int)(e & 0xFFFFu);
+        next += blockDim.x;
+      }
+      if (!__any_sync(FULL, pu >= 0)) break;
+      if (pu >= 0) {
+        int ra = pu, rb = pv;
+        pu = -1;
+        if (!s_find2(s.parent, ra, rb, cap)) {
+          ok = false;
+        } else if (ra != rb) {
+          const int hi = max(ra, rb), lo = min(ra, rb);
+          const int old = atomicMin(&s.parent[hi], lo);
+          if (old != hi && old != lo) { pu = old; pv = lo; }
+        }
       }
     }
-    __syncthreads();
-    // (no flatten between levels: path halving in s_find keeps the next
-    // level's walks short, and a full pass over all runs costs more)
   }
+  __syncthreads();
   // 4. flatten: every thread points its own runs at their roots with finds
-  // that only read.  (A path-halving find writes grandparents into the
-  // entries it passes; landing after another thread's final write to one of
-  // them, such a write would leave that run one hop short of its root.)
-  // Other threads' writes only move entries closer to the roots, so a
-  // read-only walk still ends at the root.
+  // that only read, and marks its own roots INT_MIN.  (A path-halving find
+  // writes grandparents into the entries it passes; landing after another
+  // thread's final write to one of them, such a write would leave that run
+  // one hop short of its root.)  Other threads' writes only move entries
+  // closer to the roots, so a read-only walk still ends at the root.
   {
     volatile int32_t* vp = s.parent;
     for (int i = tid; i < nruns; i += blockDim.x) {
       int x = i, it = 0;
       for (; it < cap; ++it) {
         const int q = vp[x];
-        if (q == x) break;
+        if (q == x || q < 0) break;
         if ((unsigned)q >= (unsigned)nruns) { it = cap; break; }
         x = q;
       }
       if (it == cap) { ok = false; x = i; }
-      vp[i] = x;
+      vp[i] = x == i ? INT_MIN : x;
     }
   }
   if (!ok) set_status(status, ST_INTERNAL | RS_SUNION);
   __syncthreads();
-  // roots now hold their (to be minimised) representative, encoded negative
-  for (int i = tid; i < nruns; i += blockDim.x)
-    if (s.parent[i] == i) s.parent[i] = INT_MIN;
-  __syncthreads();
   // 5. seeds: components holding a pixel of mask and N phi1
   if (phi1 != nullptr) {
-    for (int r = warp; r < g.th; r += nw) {
-      uint32_t z = warp_near_row(phi1, g.H, g.W, g.Wp, g.r0 + r, g.w0, lane, g.tww, conn);
-      z &= s.m[r][lane];
-      uint32_t zl = __shfl_up_sync(FULL, z, 1);
-      if (lane == 0) zl = 0;
-      uint32_t zs = z & ~((z << 1) | (zl >> 31));
-      while (zs) {
-        const int p = __ffs(zs) - 1;
-        zs &= zs - 1;
-        s.flag[root_of(s, sid(s, r >> 1, 32 * lane + p))] = 1;
+    for (int k = warp; k < ns; k += nw) {
+      uint32_t z = lane < g.tww ? s.sd[k][lane] : 0u;
+      const uint32_t st = s.st[k][lane];
+      const int id = s.base[k] + s.pre[k][lane] - 1;
+      while (z) {
+        const uint32_t bit = z & (0u - z);
+        z ^= bit;
+        s.flag[root_of(s, id + __popc(st & (bit | (bit - 1u))))] = 1;
       }
     }
+    // (flags are bytes and the border marks below are word atomics)
     __syncthreads();
   }
-  // 6. components on the tile border (rows 0 and th-1, first/last column)
-  for (int k = warp; k < ns; k += nw) {
-    if (lane < g.tww) {
-      for (int r = 2 * k; r <= 2 * k + 1; ++r) {
-        if (r != 0 && r != g.th - 1) continue;
-        const uint32_t m = s.m[r][lane];
-        uint32_t rs = m & ~((m << 1) | (lane > 0 ? (s.m[r][lane - 1] >> 31) : 0u));
+  // 6. components on the tile border: the run starts of the first and the
+  // last row, and the pixels of the first and the last column.  The first to
+  // mark a root lists it, and for rho gives it its border pixel as value.
+  {
+    auto claim = [&](int run, int r, int x) {
+      const int R = root_of(s, run);
+      const uint32_t bit = 2u << (8 * (R & 3));
+      const uint32_t was = atomicOr(reinterpret_cast<uint32_t*>(s.flag) + (R >> 2), bit);
+      if (was & bit) return;
+      s.pend[atomicAdd(&s.nlist, 1)] = (uint32_t)R;
+      if (phi1 != nullptr) s.parent[R] = -((g.r0 + r) * g.W + 32 * g.w0 + x + 2);
+    };
+    const int rows = g.th > 1 ? 2 : 1;
+    for (int i = tid; i < rows * g.tww + 2 * ns; i += blockDim.x) {
+      if (i < rows * g.tww) {
+        const int r = i < g.tww ? 0 : g.th - 1, w = i < g.tww ? i : i - g.tww, k = r >> 1;
+        const uint32_t m = s.m[r][w];
+        uint32_t rs = m & ~((m << 1) | (w > 0 ? (s.m[r][w - 1] >> 31) : 0u));
+        const uint32_t st = s.st[k][w];
+        const int id = s.base[k] + s.pre[k][w] - 1;
         while (rs) {
           const int p = __ffs(rs) - 1;
           rs &= rs - 1;
-          s.flag[root_of(s, sid(s, k, 32 * lane + p))] |= 2;
+          claim(id + __popc(st & le_mask(p)), r, 32 * w + p);
         }
+      } else {
+        const int j = i - rows * g.tww, k = j >> 1;
+        const int w = j & 1 ? g.tww - 1 : 0, p = j & 1 ? 31 : 0;
+        for (int r = 2 * k; r <= 2 * k + 1; ++r)
+          if ((s.m[r][w] >> p) & 1u)
+            claim(s.base[k] + s.pre[k][w] + __popc(s.st[k][w] & le_mask(p)) - 1, r, 32 * w + p);
       }
-      const uint32_t u = s.u[k][lane];
-      if (lane == 0 && (u & 1u)) s.flag[root_of(s, s.base[k])] |= 2;
-      if (lane == g.tww - 1 && (u >> 31)) s.flag[root_of(s, s.base[k + 1] - 1)] |= 2;
     }
   }
   // 7. minimum pixel of each component (for canonical labels): only strip
   // runs in the component's first strip can hold it
-  if (min_pixel) {
+  if (phi1 == nullptr) {
     for (int k = warp; k < ns; k += nw) {
       if (lane >= g.tww) continue;
       uint32_t sc = s.st[k][lane];
@@ -614,132 +676,41 @@ VL_DEV bool ccl_tile_label(CclSmem& s, const uint32_t* mask, const uint32_t* phi
     }
   }
   __syncthreads();
-  return true;
+  return nruns;
 }
 
-// Per-tile storage between the local and the final pass: the encoded
-// union-find state (non-roots: their root; roots: -(representative + 2))
-// and the component flags.  The final pass rebuilds the strips from the mask
-// and reloads this instead of labelling the tile again.
-VL_DEV int ccl_tile_cap(int Wp, int cth = CCL_TH) { return (cth / 2) * min(CCL_TWW, Wp) * 32; }
-
-VL_DEV void ccl_tile_save(const CclSmem& s, int32_t* tpar, uint8_t* tflag) {
-  for (int i = threadIdx.x; i < s.nruns; i += blockDim.x) {
-    tpar[i] = s.parent[i];
-    tflag[i] = s.flag[i];
-  }
-}
-
-VL_DEV bool ccl_tile_load(CclSmem& s, const uint32_t* mask, const CclGeom& g, int conn,
-                          const int32_t* tpar, const uint8_t* tflag, int32_t* status) {
-  const int n = ccl_tile_strips(s, mask, g, conn);
-  if (n > CCL_MAXRUNS) {
-    set_status(status, ST_INTERNAL | RS_TRUNS);
-    return false;
-  }
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    int v = ldcg(tpar + i);
-    if (v >= n) {  // never written by a successful local pass: keep indexes in range
-      set_status(status, ST_INTERNAL | RS_TLOAD);
-      v = -2;
-    }
-    s.parent[i] = v;
-    s.flag[i] = ldcg(tflag + i);
-  }
-  __syncthreads();
-  return true;
-}
-
-// Encoded value of the root of strip run i (see ccl_encode_roots).
-VL_DEV int root_value(const CclSmem& s, int i) {
-  int p = s.parent[i];
-  if (p >= 0) p = s.parent[p];
-  return -p - 2;
-}
-// Value at tile pixel (row r, column x), which must be set.
-VL_DEV int pixel_value(const CclSmem& s, int r, int x) {
-  return root_value(s, sid(s, r >> 1, x));
-}
-
-// Modes of ccl_encode_roots.
-constexpr int ENC_PUBLISH = 0;     // labels: value = minimum pixel; publish border roots
-constexpr int ENC_PUBLISH_RZ = 1;  // rho: value = key (below); publish border roots
-constexpr int ENC_LABEL = 2;       // value = global label (border roots resolved in G)
-constexpr int ENC_SELECT = 3;      // flag bit2 = component selected (rho)
-
-// Keys of the component select.  A tile-local component is keyed by the
-// first pixel v of its root strip run when it holds a seed pixel, and by
-// v + npx when it does not; G then has 2 * npx entries.  The global merge
-// links the larger root under the smaller, so a merged component's root is
-// a seeded key (< npx) exactly when one of its parts was seeded: the seed
-// flag travels with the union itself and no separate pass has to gather it.
+// Keys of the component select.  A tile-local component is keyed by a border
+// pixel v when it holds a seed pixel, and by v + npx when it does not; G then
+// has 2 * npx entries.  The global merge links the larger root under the
+// smaller, so a merged component's root is a seeded key (< npx) exactly when
+// one of its parts was seeded: the seed flag travels with the union itself
+// and no separate pass has to gather it.  (Components that do not reach the
+// tile border need no key.)
 VL_DEV int rz_key(int v, bool seeded, int npx) { return seeded ? v : v + npx; }
 
-// Give every local root its value.  The publishing modes visit each root
-// once, at its start pixel, and replace parent[root] by -(value + 2); the
-// resolving modes (ENC_LABEL, ENC_SELECT) start from the saved values and
-// walk G for the roots of border components only.  Block barrier at the end.
-//   ENC_PUBLISH     value = the component's minimum pixel (computed by the
-//                   labelling); border components publish G[value] = value
-//   ENC_PUBLISH_RZ  value = rz_key of the first pixel of the root strip run;
-//                   border components publish G[value] = value
-//   ENC_LABEL       value = the global root of the saved value (border
-//                   components), else the saved value
-//   ENC_SELECT      flag bit2 set when the component is selected: seeded
-//                   locally, or its global root is a seeded key
-// glen: entries of G (npx for labels, 2 * npx for rho).  Finds compress
-// their paths: a node only ever moves to an ancestor, and in the labelling
-// the final label of every node on a path is the root it is moved to.
-VL_DEV void ccl_encode_roots(CclSmem& s, const CclGeom& g, int mode, int32_t* G, int glen,
-                             int npx, int32_t* status) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int nw = blockDim.x >> 5;
-  const int ns = (g.th + 1) >> 1;
-  if (mode == ENC_LABEL || mode == ENC_SELECT) {
-    // the saved roots already hold their value: only the components on the
-    // tile border have work, a walk in G.  The strip runs are dealt out over
-    // every thread of the block, so the walks of one tile run side by side
-    // (the border components' roots sit in the first and last strips).
-    for (int i = threadIdx.x; i < s.nruns; i += blockDim.x) {
-      const int p = s.parent[i];
-      if (p >= 0) continue;  // not a root
-      const uint8_t fl = s.flag[i];
-      if (mode == ENC_LABEL) {
-        if (fl & 2) s.parent[i] = -(g_find(G, -p - 2, glen, status) + 2);
-      } else {
-        const bool sel = (fl & 2) ? g_find(G, -p - 2, glen, status) < npx : (fl & 1) != 0;
-        if (sel) s.flag[i] = fl | 4;
-      }
-    }
-    __syncthreads();
-    return;
-  }
-  for (int k = warp; k < ns; k += nw) {
-    if (lane >= g.tww) continue;
-    uint32_t sc = s.st[k][lane];
-    while (sc) {
-      const int p = __ffs(sc) - 1;
-      sc &= sc - 1;
-      const int x = 32 * lane + p;
-      const int S = sid(s, k, x);
-      if (s.parent[S] >= 0) continue;  // not a root
-      const uint8_t fl = s.flag[S];
-      int v;
-      if (mode == ENC_PUBLISH_RZ) {
-        v = rz_key((g.r0 + (mbit(s, 2 * k, x) ? 2 * k : 2 * k + 1)) * g.W + 32 * g.w0 + x,
-                   fl & 1, npx);
-      } else {
-        v = -s.parent[S] - 2;
-      }
-      if (fl & 2) G[v] = v;
-      s.parent[S] = -(v + 2);
-    }
-  }
-  __syncthreads();
+// The value of root R as G holds it: its key (rho) or its minimum pixel.
+VL_DEV int root_key(const CclSmem& s, int R, bool rho, int npx) {
+  const int v = -s.parent[R] - 2;
+  return rho ? rz_key(v, s.flag[R] & 1, npx) : v;
 }
 
-// Border pixels of the tile point at their component's representative in G.
-VL_DEV void ccl_publish_border(CclSmem& s, const CclGeom& g, int32_t* G) {
+// Publishes the tile's border in G: every border pixel points at its
+// component's value, and so does the value itself.  The list of border roots
+// goes to `list`: their number and that of strip runs, then value and run of
+// each.
+VL_DEV void ccl_publish(CclSmem& s, int nruns, const CclGeom& g, int32_t* G, bool rho, int npx,
+                        int32_t* list) {
+  const int nl = s.nlist;
+  for (int i = threadIdx.x; i < nl; i += blockDim.x) {
+    const int R = (int)s.pend[i], v = root_key(s, R, rho, npx);
+    G[v] = v;
+    list[2 + 2 * i] = v;
+    list[3 + 2 * i] = R;
+  }
+  if (threadIdx.x == 0) {
+    list[0] = nl;
+    list[1] = nruns;
+  }
   const int width = 32 * g.tww;
   const int n = 2 * width + 2 * g.th;
   for (int i = threadIdx.x; i < n; i += blockDim.x) {
@@ -748,19 +719,143 @@ VL_DEV void ccl_publish_border(CclSmem& s, const CclGeom& g, int32_t* G) {
     else if (i < 2 * width) { r = g.th - 1; x = i - width; }
     else if (i < 2 * width + g.th) { r = i - 2 * width; x = 0; }
     else { r = i - 2 * width - g.th; x = width - 1; }
-    if (mbit(s, r, x)) G[(g.r0 + r) * g.W + 32 * g.w0 + x] = pixel_value(s, r, x);
+    const uint32_t m = s.m[r][x >> 5];
+    if ((m >> (x & 31)) & 1u) {
+      const int v = root_key(s, root_of(s, sid(s, r >> 1, x)), rho, npx);
+      const int gid = (g.r0 + r) * g.W + 32 * g.w0 + x;
+      if (gid != v) G[gid] = v;  // (the value's own entry is written above)
+    }
   }
 }
 
-// Write labels of the tile (after ENC_LABEL).  First every strip run takes
+// Per-tile storage between the local and the final pass, in a tile's share of
+// the scratch (ccl_tile_cap entries, an int32 and a byte each).
+// Labels: s.parent of every strip run, then the list of border roots in the
+// bytes.  Rho: a 16-bit code per strip run (RzSmem) in the first half of the
+// words, the list in the second.  The final pass rebuilds the strips from
+// the mask and reloads this instead of labelling the tile again.
+VL_DEV int ccl_tile_cap(int Wp, int cth = CCL_TH) { return (cth / 2) * min(CCL_TWW, Wp) * 32; }
+
+VL_DEV void ccl_tile_save(const CclSmem& s, int nruns, int32_t* tpar) {
+  for (int i = threadIdx.x; i < nruns; i += blockDim.x) tpar[i] = s.parent[i];
+}
+VL_DEV void rz_tile_save(const CclSmem& s, int nruns, int32_t* tpar) {
+  auto code = [&](int i) -> uint32_t {
+    const int p = s.parent[i];
+    return p >= 0 ? (uint32_t)p : RZ_ROOT | ((s.flag[i] & 1) ? RZ_SEED : 0u);
+  };
+  for (int i = 2 * threadIdx.x; i < nruns; i += 2 * blockDim.x)
+    reinterpret_cast<uint32_t*>(tpar)[i >> 1] = code(i) | (i + 1 < nruns ? code(i + 1) : 0u) << 16;
+}
+
+// The final pass of labels up to the point where every root of s.parent holds
+// its component's label: the walks in G of the border roots start first, and
+// their latency passes beside the strips'.  Returns the number of strip runs
+// or -1; a block barrier at the end.
+VL_DEV int ccl_tile_load(CclSmem& s, const uint32_t* mask, const CclGeom& g, int conn,
+                         const int32_t* tpar, const int32_t* list, int cap, int32_t* G, int npx,
+                         int32_t* status) {
+  const StripRows rows = ccl_load_rows(mask, g);
+  const int2 head = __ldcg(reinterpret_cast<const int2*>(list));  // border roots, strip runs
+  const int nl = min(head.x, min(CCL_MAXBORDER, cap / 8 - 1));
+  for (int i = threadIdx.x; i < nl; i += blockDim.x) {
+    const int2 e = __ldcg(reinterpret_cast<const int2*>(list) + 1 + i);
+    s.pend[2 * i] = (uint32_t)e.y;
+    s.pend[2 * i + 1] = (uint32_t)g_find(G, e.x, npx, status);
+  }
+  const int n = __shfl_sync(FULL, ccl_tile_strips(s, rows, nullptr, g, conn), 31);
+  if (n > CCL_MAXRUNS) {
+    set_status(status, ST_INTERNAL | RS_TRUNS);
+    return -1;
+  }
+  for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    int v = ldcg(tpar + i);
+    if (v >= n) {  // never written by a successful local pass: keep indexes in range
+      set_status(status, ST_INTERNAL | RS_TLOAD);
+      v = -2;
+    }
+    s.parent[i] = v;
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < nl; i += blockDim.x) {
+    const uint32_t R = s.pend[2 * i];
+    if (R < (uint32_t)n) s.parent[R] = -((int)s.pend[2 * i + 1] + 2);
+    else set_status(status, ST_INTERNAL | RS_TLOAD);
+  }
+  __syncthreads();
+  return n;
+}
+
+// The final pass of rho: Z = the selected components of the tile.  A border
+// component is selected when its root in G is a seeded key, any other when
+// it holds a seed pixel.  cap: the tile's capacity (ccl_tile_cap).  The loads
+// of rows, codes and list are in flight together, and the walks in G start
+// before the strips are worked out.
+VL_DEV void rz_tile_select(RzSmem& s, const uint32_t* mask, const CclGeom& g, int conn,
+                           const int32_t* tpar, int cap, int32_t* G, int npx, uint32_t* Z,
+                           int32_t* status) {
+  const int tid = threadIdx.x, lane = tid & 31, k = tid >> 5;
+  const int ns = (g.th + 1) >> 1;
+  const StripRows rows = ccl_load_rows(mask, g);
+  const int32_t* list = tpar + cap / 2;
+  const int2 head = __ldcg(reinterpret_cast<const int2*>(list));  // border roots, strip runs
+  const int nl = min(head.x, min(CCL_MAXBORDER, cap / 4 - 1));
+  const int saved = min(head.y, min(CCL_MAXRUNS, cap));
+  const uint32_t* codes = reinterpret_cast<const uint32_t*>(tpar);
+  uint32_t* sc = reinterpret_cast<uint32_t*>(s.code);
+  for (int i = tid; 2 * i < saved; i += blockDim.x) cp_async4(sc + i, codes + i);
+  cp_async_commit();
+  for (int i = tid; i < nl; i += blockDim.x) {
+    const int2 e = __ldcg(reinterpret_cast<const int2*>(list) + 1 + i);
+    const bool sel = g_find(G, e.x, 2 * npx, status) < npx;
+    s.list[i] = (uint32_t)e.y | (sel ? RZ_SEL << 16 : 0u);
+  }
+  const int n = __shfl_sync(FULL, ccl_tile_strips(s, rows, nullptr, g, conn), 31);
+  cp_async_wait<0>();
+  if (n > CCL_MAXRUNS || n != saved) {  // (uniform) not the tile that was saved
+    set_status(status, ST_INTERNAL | RS_TLOAD);
+    return;
+  }
+  __syncthreads();
+  for (int i = tid; i < nl; i += blockDim.x) {
+    const uint32_t e = s.list[i], R = e & 0xFFFFu;
+    if (R >= (uint32_t)n) set_status(status, ST_INTERNAL | RS_TLOAD);
+    else if (e >> 16) s.code[R] |= RZ_SEL;
+  }
+  __syncthreads();
+  auto selected = [&](int run) {
+    uint32_t c = s.code[run];
+    if (!(c & RZ_ROOT)) c = s.code[c & (CCL_MAXRUNS - 1)];
+    return (c & (RZ_SEED | RZ_SEL)) != 0;
+  };
+  if (k < ns && lane < g.tww) {
+    const uint32_t u = s.u[k][lane], st = s.st[k][lane];
+    const int id = s.base[k] + s.pre[k][lane];
+    uint32_t f = 0, runs = st;
+    for (int j = 0; runs; ++j) {
+      const uint32_t bit = runs & (0u - runs);
+      runs ^= bit;
+      if (selected(id + j)) f |= bit;
+    }
+    // a run entering from the left word continues through bit 0
+    const uint32_t e = u & ~st;
+    const uint32_t inj = (f << 1) | ((e & 1u) && selected(id - 1) ? 1u : 0u);
+    // carry through the continuation bits of each selected run
+    const uint32_t sel = f | (((e + inj) ^ e) & e);
+    for (int r = 2 * k; r <= 2 * k + 1 && r < g.th; ++r)
+      Z[(size_t)(g.r0 + r) * g.Wp + g.w0 + lane] = s.m[r][lane] & sel;
+  }
+}
+
+// Write labels of the tile (after ccl_tile_load).  First every strip run takes
 // its root's encoded value (after the flatten non-roots point at roots, and
 // roots are not written, so the pass needs no ordering), then each lane
 // writes 4 consecutive pixels per step: a warp covers 128 pixels of a row
 // with 16-byte stores when rows are 16-byte aligned.
-VL_DEV void ccl_write_labels(CclSmem& s, const CclGeom& g, int32_t* labels) {
+VL_DEV void ccl_write_labels(CclSmem& s, int nruns, const CclGeom& g, int32_t* labels) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int nw = blockDim.x >> 5;
-  for (int i = threadIdx.x; i < s.nruns; i += blockDim.x) {
+  for (int i = threadIdx.x; i < nruns; i += blockDim.x) {
     const int p = s.parent[i];
     if (p >= 0) s.parent[i] = s.parent[p];
   }
@@ -785,30 +880,6 @@ VL_DEV void ccl_write_labels(CclSmem& s, const CclGeom& g, int32_t* labels) {
         for (int q = 0; q < 4 && x0 + q < x_end; ++q) row[x0 + q] = v[q];
       }
     }
-  }
-}
-
-// Write Z = the selected components of the tile (after ENC_SELECT).
-VL_DEV void ccl_write_select(const CclSmem& s, const CclGeom& g, uint32_t* Z) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int nw = blockDim.x >> 5;
-  const int ns = (g.th + 1) >> 1;
-  for (int k = warp; k < ns; k += nw) {
-    if (lane >= g.tww) continue;
-    const uint32_t u = s.u[k][lane], st = s.st[k][lane];
-    uint32_t f = 0, sc = st;
-    while (sc) {
-      const int p = __ffs(sc) - 1;
-      sc &= sc - 1;
-      if (s.flag[root_of(s, sid(s, k, 32 * lane + p))] & 4) f |= 1u << p;
-    }
-    // a run entering from the left word continues through bit 0
-    const uint32_t e = u & ~st;
-    const uint32_t inj = (f << 1) | ((e & 1u) && (s.flag[root_of(s, sid(s, k, 32 * lane))] & 4) ? 1u : 0u);
-    // carry through the continuation bits of each selected run
-    const uint32_t sel = f | (((e + inj) ^ e) & e);
-    for (int r = 2 * k; r <= 2 * k + 1 && r < g.th; ++r)
-      Z[(size_t)(g.r0 + r) * g.Wp + g.w0 + lane] = s.m[r][lane] & sel;
   }
 }
 

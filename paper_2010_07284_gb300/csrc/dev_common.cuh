@@ -40,6 +40,20 @@ VL_DEV uint8_t ldcg(const uint8_t* p) {
   return (uint8_t)__ldcg((const unsigned char*)p);
 }
 
+// Asynchronous copies to shared memory, in groups per thread.
+VL_DEV void cp_async4(uint32_t* smem_dst, const uint32_t* gmem_src) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(smem_dst);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(gmem_src) : "memory");
+}
+VL_DEV void cp_async16(uint32_t* smem_dst, const uint32_t* gmem_src) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(smem_dst);
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(gmem_src) : "memory");
+}
+VL_DEV void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+// Waits until at most N of this thread's latest copy groups are unfinished.
+template <int N>
+VL_DEV void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
 // First error wins.
 VL_DEV void set_status(int32_t* status, int code) {
   if (status) atomicCAS(status, 0, code);

@@ -35,13 +35,6 @@ struct GroupCtx {
   int rank_mask, rank_halo;
 };
 
-VL_DEV void cp_async4(uint32_t* smem_dst, const uint32_t* gmem_src) {
-  const unsigned d = (unsigned)__cvta_generic_to_shared(smem_dst);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(gmem_src) : "memory");
-}
-VL_DEV void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-VL_DEV void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-
 // Words of the stage that the planes of the group's rank tables take (rows
 // of the core tile plus rank_halo above and below, all buffer words).
 VL_DEV int rank_stage_words(const GroupCtx& c, int upto_table) {
@@ -128,7 +121,7 @@ VL_DEV void group_tile_t(const GroupCtx& c, const Insn* insns, int n_insn) {
     const int w_lo = i_lo * bw, w_hi = i_hi * bw;           // buffer words
     if (op == I_RTHR) {
       if (stage == 1) {  // uniform: every thread waits for its copies, then all
-        cp_async_wait_all();
+        cp_async_wait<0>();
         __syncthreads();
         stage = 2;
       }
@@ -307,7 +300,7 @@ VL_DEV void group_tile_t(const GroupCtx& c, const Insn* insns, int n_insn) {
       }
     }
   }
-  if (stage == 1) cp_async_wait_all();  // no copy may outlive the tile
+  if (stage == 1) cp_async_wait<0>();  // no copy may outlive the tile
 }
 
 // The group interpreter for the tile widths the autotuner tries (buffer

@@ -184,24 +184,21 @@ VL_DEV void run_subitem(const DevJob& J, const StepDesc& S, int sub, int per_rz,
       break;
     case SK_RZ_LOCAL:
     case SK_RZ_FINAL: {
-      CclSmem& s = *reinterpret_cast<CclSmem*>(smem);
       const int j = sub / per_rz, tile = sub - j * per_rz;
       const RzDesc r = J.rz[S.rz_off + j];
       const int k = r.scratch;
       const CclGeom geo = ccl_geom(J.H, J.W, J.Wp, tile, J.c_tiles_x, J.H, J.c_th);
-      const uint32_t* phi1 = J.slots[r.phi1_slot];
       const uint32_t* phi2 = J.slots[r.phi2_slot];
-      int32_t* tpar = rz_tpar(J, k) + (size_t)tile * J.tile_cap;
-      uint8_t* tflag = rz_tflag(J, k) + (size_t)tile * J.tile_cap;
+      int32_t* state = rz_state(J, k) + (size_t)tile * J.tile_cap;
       if (S.kind == SK_RZ_LOCAL) {
-        if (!ccl_tile_label(s, phi2, phi1, geo, J.conn, false, J.status)) break;
-        ccl_encode_roots(s, geo, ENC_PUBLISH_RZ, rz_G(J, k), 2 * npx, npx, J.status);
-        ccl_publish_border(s, geo, rz_G(J, k));
-        ccl_tile_save(s, tpar, tflag);
+        CclSmem& s = *reinterpret_cast<CclSmem*>(smem);
+        const int nruns = ccl_tile_label(s, phi2, J.slots[r.phi1_slot], geo, J.conn, J.status);
+        if (nruns < 0) break;
+        ccl_publish(s, nruns, geo, rz_G(J, k), true, npx, state + J.tile_cap / 2);
+        rz_tile_save(s, nruns, state);
       } else {
-        if (!ccl_tile_load(s, phi2, geo, J.conn, tpar, tflag, J.status)) break;
-        ccl_encode_roots(s, geo, ENC_SELECT, rz_G(J, k), 2 * npx, npx, J.status);
-        ccl_write_select(s, geo, J.slots[r.z_slot]);
+        rz_tile_select(*reinterpret_cast<RzSmem*>(smem), phi2, geo, J.conn, state, J.tile_cap,
+                       rz_G(J, k), npx, J.slots[r.z_slot], J.status);
       }
       break;
     }

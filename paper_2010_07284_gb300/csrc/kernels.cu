@@ -238,20 +238,21 @@ __global__ void k_arith(int op, const void* __restrict__ a, int a_format, const 
 
 // ------------------------------------------------------------------ ccl --
 
+// phi1 null: full labelling (canonical minimum pixels), else the select of rho.
 __global__ void __launch_bounds__(EXEC_THREADS, 2)
 k_ccl_local(const uint32_t* mask, const uint32_t* phi1, MaskGeom g, int tiles_x, int conn,
             CclScratch sc, int32_t* status) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   CclSmem& s = *reinterpret_cast<CclSmem*>(smem_raw);
   const CclGeom geo = ccl_geom(g.H, g.W, g.Wp, blockIdx.x, tiles_x, slice_rows(g), ccl_rows(g));
-  const int npx = g.H * g.W;
-  const bool labels = phi1 == nullptr;  // full labelling: canonical minimum pixel
-  if (!ccl_tile_label(s, mask, phi1, geo, conn, labels, status)) return;
-  ccl_encode_roots(s, geo, labels ? ENC_PUBLISH : ENC_PUBLISH_RZ, sc.G, labels ? npx : 2 * npx,
-                   npx, status);
-  ccl_publish_border(s, geo, sc.G);
-  ccl_tile_save(s, sc.tpar + (size_t)blockIdx.x * sc.tile_cap,
-                sc.tflag + (size_t)blockIdx.x * sc.tile_cap);
+  const bool rho = phi1 != nullptr;
+  const int nruns = ccl_tile_label(s, mask, phi1, geo, conn, status);
+  if (nruns < 0) return;
+  int32_t* state = sc.tpar + (size_t)blockIdx.x * sc.tile_cap;
+  ccl_publish(s, nruns, geo, sc.G, rho, g.H * g.W,
+              rho ? state + sc.tile_cap / 2 : tile_list(sc, blockIdx.x));
+  if (rho) rz_tile_save(s, nruns, state);
+  else ccl_tile_save(s, nruns, state);
 }
 
 // glen: entries of G (H*W for labels, 2*H*W for rho keys).
@@ -270,26 +271,18 @@ k_ccl_final_labels(const uint32_t* mask, MaskGeom g, int tiles_x, int conn, CclS
   extern __shared__ __align__(16) unsigned char smem_raw[];
   CclSmem& s = *reinterpret_cast<CclSmem*>(smem_raw);
   const CclGeom geo = ccl_geom(g.H, g.W, g.Wp, blockIdx.x, tiles_x, slice_rows(g), ccl_rows(g));
-  const int npx = g.H * g.W;
-  if (!ccl_tile_load(s, mask, geo, conn, sc.tpar + (size_t)blockIdx.x * sc.tile_cap,
-                     sc.tflag + (size_t)blockIdx.x * sc.tile_cap, status))
-    return;
-  ccl_encode_roots(s, geo, ENC_LABEL, sc.G, npx, npx, status);
-  ccl_write_labels(s, geo, sc.G);
+  const int nruns = ccl_tile_load(s, mask, geo, conn, sc.tpar + (size_t)blockIdx.x * sc.tile_cap,
+                                  tile_list(sc, blockIdx.x), sc.tile_cap, sc.G, g.H * g.W, status);
+  if (nruns >= 0) ccl_write_labels(s, nruns, geo, sc.G);
 }
 
-__global__ void __launch_bounds__(EXEC_THREADS, 2)
-k_rz_final(const uint32_t* phi1, const uint32_t* phi2, MaskGeom g, int tiles_x, int conn,
-           CclScratch sc, uint32_t* Z, int32_t* status) {
+__global__ void __launch_bounds__(EXEC_THREADS, 3)
+k_rz_final(const uint32_t* phi2, MaskGeom g, int tiles_x, int conn, CclScratch sc, uint32_t* Z,
+           int32_t* status) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  CclSmem& s = *reinterpret_cast<CclSmem*>(smem_raw);
   const CclGeom geo = ccl_geom(g.H, g.W, g.Wp, blockIdx.x, tiles_x, slice_rows(g), ccl_rows(g));
-  const int npx = g.H * g.W;
-  if (!ccl_tile_load(s, phi2, geo, conn, sc.tpar + (size_t)blockIdx.x * sc.tile_cap,
-                     sc.tflag + (size_t)blockIdx.x * sc.tile_cap, status))
-    return;
-  ccl_encode_roots(s, geo, ENC_SELECT, sc.G, 2 * npx, npx, status);
-  ccl_write_select(s, geo, Z);
+  rz_tile_select(*reinterpret_cast<RzSmem*>(smem_raw), phi2, geo, conn,
+                 sc.tpar + (size_t)blockIdx.x * sc.tile_cap, sc.tile_cap, sc.G, g.H * g.W, Z, status);
 }
 
 // ----------------------------------------------------------- conversion --
@@ -445,7 +438,8 @@ static cudaError_t ccl_set_attrs() {
   if ((e = cudaFuncSetAttribute(k_ccl_final_labels,
                                 cudaFuncAttributeMaxDynamicSharedMemorySize, sm)))
     return e;
-  if ((e = cudaFuncSetAttribute(k_rz_final, cudaFuncAttributeMaxDynamicSharedMemorySize, sm)))
+  if ((e = cudaFuncSetAttribute(k_rz_final, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)sizeof(RzSmem))))
     return e;
   g_attr_done[dev] = true;
   return cudaSuccess;
@@ -491,7 +485,7 @@ cudaError_t launch_rz(const uint32_t* phi1, const uint32_t* phi2, MaskGeom g, in
                                                              2 * g.H * g.W, status);
     if ((e = cudaGetLastError())) return e;
   }
-  k_rz_final<<<ty * tx, EXEC_THREADS, sm, st>>>(phi1, phi2, g, tx, conn, sc, Z, status);
+  k_rz_final<<<ty * tx, EXEC_THREADS, sizeof(RzSmem), st>>>(phi2, g, tx, conn, sc, Z, status);
   return cudaGetLastError();
 }
 

@@ -49,9 +49,12 @@ struct CclScratch {
                     // itself), 2*H*W for rho (pixel ids, then the keys of
                     // unseeded components)
   int32_t tile_cap; // per-tile capacity of tpar / tflag (ccl_tile_cap_host)
-  int32_t* tpar;    // tiles * tile_cap int32: saved tile union-find state
-  uint8_t* tflag;   // tiles * tile_cap bytes: saved tile flags
+  int32_t* tpar;    // tiles * tile_cap int32: saved tile state
+  uint8_t* tflag;   // tiles * tile_cap bytes: lists of border roots (labels only)
 };
+inline __host__ __device__ int32_t* tile_list(const CclScratch& sc, int tile) {
+  return reinterpret_cast<int32_t*>(sc.tflag + (size_t)tile * sc.tile_cap);
+}
 // Labelling tiles: rows over all slices (Hs 0: an image; cth: rows per
 // tile, even, at most CCL_TH), columns, per-tile saved-state capacity.
 int ccl_tiles_y(int H, int Hs = 0, int cth = CCL_TH);

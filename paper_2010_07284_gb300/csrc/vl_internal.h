@@ -23,8 +23,16 @@ constexpr int CCL_NS = CCL_TH / 2;
 // A strip run can start at every column under 4-adjacency (checkerboard).
 constexpr int CCL_MAXRUNS = CCL_NS * CCL_TWW * 32;
 
+// Components of a tile that reach its border: at most one per row-run start
+// of the first and the last row and per pixel of the outer columns.
+constexpr int CCL_MAXBORDER = 2 * CCL_TWW * 16 + 2 * CCL_TH;
+
 constexpr int EXEC_THREADS = 512;  // threads per CTA of every tiled kernel
 constexpr int EXEC_WARPS = EXEC_THREADS / 32;
+
+// Shared memory that a context sets aside for the buffers of group tiles (14
+// buffers of a 32 x 32-word tile with 8 halo rows above and below).
+constexpr int kGroupBudget = 14 * 48 * 34 * 4;
 
 // Device status word values (match vl_status where they overlap).
 constexpr int ST_OK = 0;
@@ -198,11 +206,10 @@ struct DevJob {
   float* pct_val;               // percentile values by slot
   // CCL scratch sets, one per select of a batch step, `set_bytes` apart:
   // union-find over keys (G, 2 * H * W entries: pixel ids and the keys of
-  // unseeded components), saved tile union-find state and flags (tiles x
-  // tile_cap)
+  // unseeded components), saved tile state (tiles x tile_cap words)
   unsigned char* rzs;
   int64_t set_bytes;
-  int64_t off_tpar, off_tflag;
+  int64_t off_state;
   int32_t tile_cap;
   int32_t c_th;                 // rows of a labelling tile (16 or 32)
   int32_t* status;              // device status word of this job
@@ -219,10 +226,9 @@ struct DevJob {
 VL_HD_INLINE int32_t* rz_G(const DevJob& J, int k) {
   return reinterpret_cast<int32_t*>(J.rzs + k * J.set_bytes);
 }
-VL_HD_INLINE int32_t* rz_tpar(const DevJob& J, int k) {
-  return reinterpret_cast<int32_t*>(J.rzs + k * J.set_bytes + J.off_tpar);
+VL_HD_INLINE int32_t* rz_state(const DevJob& J, int k) {
+  return reinterpret_cast<int32_t*>(J.rzs + k * J.set_bytes + J.off_state);
 }
-VL_HD_INLINE uint8_t* rz_tflag(const DevJob& J, int k) { return J.rzs + k * J.set_bytes + J.off_tflag; }
 
 // One work item of the persistent executor: a range of `count` consecutive
 // sub-items (tiles, chunks, rz x tile) of one step of one job.
