@@ -421,6 +421,14 @@ vl_status batch_build(vl_context* ctx, const vl_job* jobs, int n_jobs, cudaStrea
   for (size_t k = 0; k < formulas.size(); ++k) {
     const Plan* P = formulas[k];
     if (!P->steps.empty()) std::memcpy(&host[f_steps[k]], P->steps.data(), sizeof(StepDesc) * P->steps.size());
+    // on the device a group's pct_cnt counts its float thresholds, pct_off its loads
+    StepDesc* hs = reinterpret_cast<StepDesc*>(&host[f_steps[k]]);
+    for (size_t q = 0; q < P->steps.size(); ++q)
+      for (int i = 0; hs[q].kind == SK_GROUP && i < hs[q].insn_cnt; ++i) {
+        const int op = insn_op(P->insns[hs[q].insn_off + i]);
+        hs[q].pct_cnt += op == I_THR;
+        hs[q].pct_off += op == I_LOAD;
+      }
     if (!P->insns.empty()) std::memcpy(&host[f_insns[k]], P->insns.data(), sizeof(Insn) * P->insns.size());
     if (!P->rz.empty()) std::memcpy(&host[f_rz[k]], P->rz.data(), sizeof(RzDesc) * P->rz.size());
     if (!P->pct.empty()) std::memcpy(&host[f_pct[k]], P->pct.data(), sizeof(PctDesc) * P->pct.size());
@@ -468,6 +476,10 @@ vl_status batch_build(vl_context* ctx, const vl_job* jobs, int n_jobs, cudaStrea
     for (int s = 0; s < P.n_mask_slots; ++s)
       hs[P.n_inter_slots + P.n_root_slots + s] = jobs[j].images[P.mask_slot_image[s]]->mask;
     d.slots = reinterpret_cast<uint32_t* const*>(tb + I.off_slotptrs);
+    d.slot_mem = reinterpret_cast<uint32_t*>(tb + I.off_slots);
+    d.root_mem = reinterpret_cast<uint32_t*>(pb + I.off_roots);
+    d.n_inter_slots = P.n_inter_slots;
+    d.n_root_slots = P.n_root_slots;
     const int k = I.formula_idx;
     d.insns = reinterpret_cast<const Insn*>(tb + f_insns[k]);
     d.steps = reinterpret_cast<const StepDesc*>(tb + f_steps[k]);
@@ -507,8 +519,6 @@ vl_status batch_build(vl_context* ctx, const vl_job* jobs, int n_jobs, cudaStrea
   L.need = reinterpret_cast<const int32_t*>(tb + off_need);
   L.spin_limit = ctx->cfg.spin_limit != 0 ? ctx->cfg.spin_limit : (1LL << 22);
   L.group_buffers = ctx->nb;
-  L.group_bh = ts.rows + 2 * ctx->hmax;
-  L.group_bw = ts.words + 2;
   L.grid = std::max(1, std::min<int>(grid, (int)items.size()));
   L.smem_bytes = (int32_t)ctx->exec_smem;
   L.trace = nullptr;
@@ -974,13 +984,12 @@ VL_API vl_status vl_context_create(const vl_config* cfg, vl_context** out) {
   c->gth = c->cfg.tile_rows > 0 ? c->cfg.tile_rows : 32;
   c->gtww = c->cfg.tile_words > 0 ? c->cfg.tile_words : 32;
   c->hmax = 8;
-  const int bh = c->gth + 2 * c->hmax, bw = c->gtww + 2;
-  const size_t budget = kGroupBudget;
-  c->nb = (int)std::min<size_t>(64, budget / ((size_t)bh * bw * 4));
+  const int bh = c->gth + 2 * c->hmax;
+  c->nb = (int)std::min<int64_t>(64, kGroupBudget / group_buffer_bytes(bh, c->gtww));
   if (c->nb < 4) { delete c; return VL_ERR_ARG; }
   c->pp.group_buffers = c->nb;
   c->pp.hmax = c->hmax;
-  c->exec_smem = exec_smem_bytes(c->nb, bh, bw);
+  c->exec_smem = exec_smem_bytes(c->nb, bh, c->gtww);
   {
     // room beside the group buffers for staging rank planes, as long as two
     // CTAs still fit on an SM
@@ -991,14 +1000,14 @@ VL_API vl_status vl_context_create(const vl_config* cfg, vl_context** out) {
       cudaGetLastError();
     } else {
       // (less the executor's static shared words and some slack)
-      const size_t two = ((size_t)(smem_sm / 2 - reserved - 256)) & ~(size_t)127;
+      const size_t two = ((size_t)(smem_sm / 2 - reserved - 1024)) & ~(size_t)127;
       if (two > c->exec_smem && two <= (size_t)optin) c->exec_smem = two;
     }
   }
   if ((e = exec_configure(c->exec_smem, &c->ctas_per_sm))) { delete c; cudaGetLastError(); return VL_ERR_CUDA; }
-  if (c->ctas_per_sm < 2 && c->exec_smem > exec_smem_bytes(c->nb, bh, bw)) {
+  if (c->ctas_per_sm < 2 && c->exec_smem > exec_smem_bytes(c->nb, bh, c->gtww)) {
     // the widened size lost the second CTA on this GPU: fall back
-    c->exec_smem = exec_smem_bytes(c->nb, bh, bw);
+    c->exec_smem = exec_smem_bytes(c->nb, bh, c->gtww);
     if ((e = exec_configure(c->exec_smem, &c->ctas_per_sm))) { delete c; cudaGetLastError(); return VL_ERR_CUDA; }
   }
   if (c->ctas_per_sm < 1) c->ctas_per_sm = 1;
@@ -1256,9 +1265,7 @@ static PlanParams default_plan_params() {
   // halo budget 8, buffers that fit the labelling footprint
   PlanParams pp;
   pp.hmax = 8;
-  const int bh = 32 + 2 * pp.hmax, bw = 32 + 2;
-  const size_t budget = kGroupBudget;
-  pp.group_buffers = (int)std::min<size_t>(64, budget / ((size_t)bh * bw * 4));
+  pp.group_buffers = (int)(kGroupBudget / group_buffer_bytes(32 + 2 * pp.hmax, 32));
   return pp;
 }
 

@@ -100,8 +100,9 @@ uint64_t plan_hash(const Plan& P) {
 
 bool tile_shape_fits(const vl_context* ctx, const TileShape& t) {
   if (t.rows < 1 || t.words < 1) return false;
-  const size_t bytes = (size_t)ctx->nb * (t.rows + 2 * ctx->hmax) * (t.words + 2) * 4;
-  return bytes <= ctx->exec_smem;
+  const int64_t bytes =
+      GROUP_PROG_BYTES + ctx->nb * group_buffer_bytes(t.rows + 2 * ctx->hmax, t.words);
+  return bytes <= (int64_t)ctx->exec_smem;
 }
 
 TileShape pick_tile_shape(vl_context* ctx, const vl_job* jobs, int n_jobs, int* tuned,

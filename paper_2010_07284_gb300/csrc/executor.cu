@@ -33,6 +33,20 @@ VL_DEV int ld_acquire(const int32_t* p) {
   return v;
 }
 
+// Thread 0 polls *ctr with back-off until it is at least `need`; false when
+// the limit runs out first (a negative one does at once).
+VL_DEV bool poll_count(const int32_t* ctr, int need, long long spin_limit, const int32_t* status) {
+  long long spins = 0;
+  unsigned ns = 32;
+  if (spin_limit < 0) return false;
+  while (ld_acquire(ctr) < need) {
+    if (++spins > spin_limit || (status && ldcg(status) != 0)) return false;
+    __nanosleep(ns);
+    if (ns < 1024) ns <<= 1;
+  }
+  return true;
+}
+
 // Rank codes of rows [y0, y1) of one channel against the sorted table tv
 // (see RankTab): one warp per 32-pixel word, one lane per pixel; code bit b
 // of the word's pixels is a ballot, written to plane b (lane b writes it).
@@ -131,142 +145,166 @@ VL_DEV void arith_rows(const DevJob& J, int sub, unsigned char* smem) {
   }
 }
 
-VL_DEV void run_subitem(const DevJob& J, const StepDesc& S, int sub, int per_rz,
-                        unsigned char* smem, const ExecLaunch& L) {
+// The executor's dynamic shared memory, by name: through a pointer argument
+// its accesses would be generic ones.
+extern __shared__ __align__(16) unsigned char exec_smem[];
+// The job and the step of the item at hand (read by every sub-item; from
+// global memory each of their fields is a dependent access of its own).
+__shared__ DevJob s_job;
+__shared__ StepDesc s_step;
+static_assert(sizeof(DevJob) % 8 == 0 && sizeof(StepDesc) <= 128, "copied by one warp");
+
+// The kinds of sub-items, each a function of its own: the registers of one
+// then do not depend on what the others keep alive (inlined into one kernel
+// at 64 registers a thread, the interpreter's loop spilled).
+
+__device__ __noinline__ void percentile_item(int sub) {
+  const DevJob& J = s_job;
+  const StepDesc& S = s_step;
+  SelectSmem& s = *reinterpret_cast<SelectSmem*>(exec_smem);
+  const PctDesc d = J.pct[S.pct_off + sub];
+  const DevImage im = J.images[d.img];
+  const long long n = (long long)J.H * J.W;
+  const long long rank = (long long)(d.q * (double)(n - 1));
+  const float v = select_rank(s, chan_ptr(im, d.ch, (size_t)J.H * J.pitch), im.format, !im.written,
+                              J.H, J.W, J.pitch, rank);
+  if (threadIdx.x == 0) J.pct_val[d.slot] = v;
+}
+
+__device__ __noinline__ void group_item(int sub, const ExecLaunch& L) {
+  const DevJob& J = s_job;
+  const StepDesc& S = s_step;
+  group_tile(J, S, sub, reinterpret_cast<uint32_t*>(exec_smem), L.smem_bytes / 4, L.group_buffers);
+}
+
+__device__ __noinline__ void rank_item(int sub) {
+  const DevJob& J = s_job;
+  const int per_tab = (J.H + RANK_ROWS - 1) / RANK_ROWS;
+  const int tab = sub / per_tab, rb = sub - tab * per_tab;
+  const RankTab T = J.rtab[tab];
+  float* tv = reinterpret_cast<float*>(exec_smem);
+  for (int i = threadIdx.x; i < T.m; i += blockDim.x) tv[i] = J.rvals[T.val_off + i];
+  __syncthreads();
+  const DevImage im = J.images[T.img];
+  rank_rows(tv, T, chan_ptr(im, T.ch, (size_t)J.H * J.pitch), im.format, !im.written, J.H,
+            J.W, J.Wp, J.pitch, rb * RANK_ROWS, min(J.H, (rb + 1) * RANK_ROWS),
+            J.planes + (size_t)T.plane0 * J.H * J.Wp);
+}
+
+__device__ __noinline__ void arith_item(int sub) {
+  arith_rows(s_job, sub, exec_smem);
+}
+
+__device__ __noinline__ void rz_local_item(int sub, int per_rz) {
+  const DevJob& J = s_job;
+  const StepDesc& S = s_step;
   const int npx = J.H * J.W;
-  switch (S.kind) {
-    case SK_PCT: {
-      SelectSmem& s = *reinterpret_cast<SelectSmem*>(smem);
-      const PctDesc d = J.pct[S.pct_off + sub];
-      const DevImage im = J.images[d.img];
-      const long long n = (long long)J.H * J.W;
-      const long long rank = (long long)(d.q * (double)(n - 1));
-      const float v = select_rank(s, chan_ptr(im, d.ch, (size_t)J.H * J.pitch), im.format,
-                                  !im.written, J.H, J.W, J.pitch, rank);
-      if (threadIdx.x == 0) J.pct_val[d.slot] = v;
-      break;
-    }
-    case SK_GROUP: {
-      GroupCtx c;
-      c.H = J.H; c.W = J.W; c.Wp = J.Wp; c.pitch = J.pitch;
-      const int ty = sub / J.g_tiles_x, tx = sub - ty * J.g_tiles_x;
-      c.r0 = ty * J.gth; c.w0 = tx * J.gtww;
-      c.th = min(J.gth, J.H - c.r0); c.tww = min(J.gtww, J.Wp - c.w0);
-      c.halo = S.halo;
-      c.bh = L.group_bh; c.bw = L.group_bw;
-      c.conn = J.conn;
-      c.buf = reinterpret_cast<uint32_t*>(smem);
-      c.images = J.images; c.slots = J.slots; c.pct_val = J.pct_val;
-      c.rtab = J.rtab; c.planes = J.planes; c.pstride = (size_t)J.H * J.Wp;
-      // the stage of rank planes follows the buffers this group uses
-      const int nbuf = min(max(S.n_bufs, 1), L.group_buffers);
-      c.stage = c.buf + (size_t)nbuf * c.bh * c.bw;
-      c.stage_cap = L.smem_bytes / 4 - nbuf * c.bh * c.bw;
-      c.rank_mask = S.rank_mask; c.rank_halo = S.rank_halo;
-      group_tile(c, J.insns + S.insn_off, S.insn_cnt);
-      break;
-    }
-    case SK_RANK: {
-      const int per_tab = (J.H + RANK_ROWS - 1) / RANK_ROWS;
-      const int tab = sub / per_tab, rb = sub - tab * per_tab;
-      const RankTab T = J.rtab[tab];
-      float* tv = reinterpret_cast<float*>(smem);
-      for (int i = threadIdx.x; i < T.m; i += blockDim.x) tv[i] = J.rvals[T.val_off + i];
-      __syncthreads();
-      const DevImage im = J.images[T.img];
-      rank_rows(tv, T, chan_ptr(im, T.ch, (size_t)J.H * J.pitch), im.format, !im.written, J.H,
-                J.W, J.Wp, J.pitch, rb * RANK_ROWS, min(J.H, (rb + 1) * RANK_ROWS),
-                J.planes + (size_t)T.plane0 * J.H * J.Wp);
-      break;
-    }
-    case SK_ARITH:
-      arith_rows(J, sub, smem);
-      break;
-    case SK_RZ_LOCAL:
-    case SK_RZ_FINAL: {
-      const int j = sub / per_rz, tile = sub - j * per_rz;
-      const RzDesc r = J.rz[S.rz_off + j];
-      const int k = r.scratch;
-      const CclGeom geo = ccl_geom(J.H, J.W, J.Wp, tile, J.c_tiles_x, J.H, J.c_th);
-      const uint32_t* phi2 = J.slots[r.phi2_slot];
-      int32_t* state = rz_state(J, k) + (size_t)tile * J.tile_cap;
-      if (S.kind == SK_RZ_LOCAL) {
-        CclSmem& s = *reinterpret_cast<CclSmem*>(smem);
-        const int nruns = ccl_tile_label(s, phi2, J.slots[r.phi1_slot], geo, J.conn, J.status);
-        if (nruns < 0) break;
-        ccl_publish(s, nruns, geo, rz_G(J, k), true, npx, state + J.tile_cap / 2);
-        rz_tile_save(s, nruns, state);
-      } else {
-        rz_tile_select(*reinterpret_cast<RzSmem*>(smem), phi2, geo, J.conn, state, J.tile_cap,
-                       rz_G(J, k), npx, J.slots[r.z_slot], J.status);
-      }
-      break;
-    }
-    case SK_RZ_MERGE: {
-      const int j = sub / per_rz, chunk = sub - j * per_rz;
-      const RzDesc r = J.rz[S.rz_off + j];
-      const int n = merge_units(J.H, J.Wp, J.c_tiles_x, J.H, J.c_th);
-      const int nw = blockDim.x >> 5;
-      for (int u = chunk * nw + (threadIdx.x >> 5); u < n; u += per_rz * nw)
-        ccl_merge_unit(J.slots[r.phi2_slot], J.H, J.W, J.Wp, u, J.conn, rz_G(J, r.scratch),
-                       2 * npx, J.status, J.H, J.c_th);
-      break;
-    }
-    default:
-      break;
+  CclSmem& s = *reinterpret_cast<CclSmem*>(exec_smem);
+  const int j = sub / per_rz, tile = sub - j * per_rz;
+  const RzDesc r = J.rz[S.rz_off + j];
+  const int k = r.scratch;
+  const CclGeom geo = ccl_geom(J.H, J.W, J.Wp, tile, J.c_tiles_x, J.H, J.c_th);
+  const int nruns = ccl_tile_label(s, slot_ptr(J, r.phi2_slot), slot_ptr(J, r.phi1_slot), geo, J.conn,
+                                   J.status);
+  if (nruns < 0) return;
+  int32_t* state = rz_state(J, k) + (size_t)tile * J.tile_cap;
+  ccl_publish(s, nruns, geo, rz_G(J, k), true, npx, state + J.tile_cap / 2);
+  rz_tile_save(s, nruns, state);
+}
+
+__device__ __noinline__ void rz_final_item(int sub, int per_rz) {
+  const DevJob& J = s_job;
+  const StepDesc& S = s_step;
+  const int npx = J.H * J.W;
+  const int j = sub / per_rz, tile = sub - j * per_rz;
+  const RzDesc r = J.rz[S.rz_off + j];
+  const int k = r.scratch;
+  const CclGeom geo = ccl_geom(J.H, J.W, J.Wp, tile, J.c_tiles_x, J.H, J.c_th);
+  rz_tile_select(*reinterpret_cast<RzSmem*>(exec_smem), slot_ptr(J, r.phi2_slot), geo, J.conn,
+                 rz_state(J, k) + (size_t)tile * J.tile_cap, J.tile_cap, rz_G(J, k), npx,
+                 slot_ptr(J, r.z_slot), J.status);
+}
+
+__device__ __noinline__ void rz_merge_item(int sub, int per_rz) {
+  const DevJob& J = s_job;
+  const StepDesc& S = s_step;
+  const int npx = J.H * J.W;
+  const int j = sub / per_rz, chunk = sub - j * per_rz;
+  const RzDesc r = J.rz[S.rz_off + j];
+  const uint32_t* phi2 = slot_ptr(J, r.phi2_slot);
+  const int n = merge_units(J.H, J.Wp, J.c_tiles_x, J.H, J.c_th);
+  const int nw = blockDim.x >> 5;
+  for (int u = chunk * nw + (threadIdx.x >> 5); u < n; u += per_rz * nw)
+    ccl_merge_unit(phi2, J.H, J.W, J.Wp, u, J.conn, rz_G(J, r.scratch),
+                   2 * npx, J.status, J.H, J.c_th);
+}
+
+VL_DEV void run_subitem(int sub, int per_rz, const ExecLaunch& L) {
+  switch (s_step.kind) {
+    case SK_PCT: percentile_item(sub); break;
+    case SK_GROUP: group_item(sub, L); break;
+    case SK_RANK: rank_item(sub); break;
+    case SK_ARITH: arith_item(sub); break;
+    case SK_RZ_LOCAL: rz_local_item(sub, per_rz); break;
+    case SK_RZ_MERGE: rz_merge_item(sub, per_rz); break;
+    case SK_RZ_FINAL: rz_final_item(sub, per_rz); break;
+    default: break;
   }
 }
 
-__global__ void __launch_bounds__(EXEC_THREADS, 2) k_exec(ExecLaunch L) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ int s_item, s_skip;
+__global__ void __launch_bounds__(EXEC_THREADS, 2) k_exec(const __grid_constant__ ExecLaunch L) {
+  __shared__ WorkItem s_item;
+  __shared__ int s_go;  // -1: no more items, 0: skip, 1: run
   for (;;) {
-    if (threadIdx.x == 0) s_item = atomicAdd(L.head, 1);
-    __syncthreads();
-    const int idx = s_item;
-    if (idx >= L.n_items) break;
-    const WorkItem it = L.items[idx];
-    const DevJob& J = L.jobs[it.job];
-    const StepDesc S = J.steps[it.step];
-    const int ci = J.step_base + it.step;
     unsigned long long t_pop = 0, t_go = 0;
-    if (threadIdx.x == 0) {
-      if (L.trace) t_pop = now_ns();
-      int skip = 0;
-      const int d0 = J.dep_off[it.step], d1 = J.dep_off[it.step + 1];
-      // a negative limit makes every wait expire at once (tests of the
-      // timeout path); otherwise poll with back-off up to the limit
-      if (d1 > d0 && L.spin_limit < 0) {
-        set_status(J.status, ST_TIMEOUT);
-        skip = 1;
-      }
-      for (int q = d0; q < d1 && !skip; ++q) {
-        const int dep = J.step_base + J.deps[q];
-        const int32_t* ctr = L.done + dep;
-        const int need = L.need[dep];
-        long long spins = 0;
-        unsigned ns = 32;
-        while (ld_acquire(ctr) < need) {
-          if (++spins > L.spin_limit) {
-            set_status(J.status, ST_TIMEOUT);
-            skip = 1;
-            break;
+    if (threadIdx.x < 32) {
+      // warp 0 pops an item, brings its job and step to shared memory and
+      // waits for the steps the item depends on
+      const int lane = threadIdx.x;
+      int idx = 0;
+      if (lane == 0) idx = atomicAdd(L.head, 1);
+      idx = __shfl_sync(FULL, idx, 0);
+      if (idx >= L.n_items) {
+        if (lane == 0) s_go = -1;
+      } else {
+        const WorkItem it = L.items[idx];
+        const unsigned long long* src = reinterpret_cast<const unsigned long long*>(L.jobs + it.job);
+        for (int k = lane; k < (int)(sizeof(DevJob) / 8); k += 32)
+          reinterpret_cast<unsigned long long*>(&s_job)[k] = __ldg(src + k);
+        __syncwarp();
+        const int* step = reinterpret_cast<const int*>(s_job.steps + it.step);
+        if (lane < (int)(sizeof(StepDesc) / 4))
+          reinterpret_cast<int*>(&s_step)[lane] = __ldg(step + lane);
+        if (lane == 0) {
+          s_item = it;
+          if (L.trace) t_pop = now_ns();
+          int go = 1;
+          const int d0 = __ldg(s_job.dep_off + it.step), d1 = __ldg(s_job.dep_off + it.step + 1);
+          // (a negative limit makes every wait expire at once: tests of the
+          // timeout path)
+          for (int q = d0; q < d1 && go; ++q) {
+            const int dep = s_job.step_base + __ldg(s_job.deps + q);
+            if (!poll_count(L.done + dep, __ldg(L.need + dep), L.spin_limit, nullptr)) {
+              set_status(s_job.status, ST_TIMEOUT);
+              go = 0;
+            }
           }
-          __nanosleep(ns);
-          if (ns < 1024) ns <<= 1;
+          if (ldcg(s_job.status) != 0) go = 0;
+          s_go = go;
+          if (L.trace) t_go = now_ns();
         }
       }
-      if (ldcg(J.status) != 0) skip = 1;
-      s_skip = skip;
-      if (L.trace) t_go = now_ns();
     }
     __syncthreads();
-    if (!s_skip) {
+    if (s_go < 0) break;
+    const WorkItem it = s_item;
+    const int ci = s_job.step_base + it.step;
+    if (s_go) {
       int per_rz = 1;
-      if (S.kind == SK_RZ_LOCAL || S.kind == SK_RZ_MERGE || S.kind == SK_RZ_FINAL)
-        per_rz = L.need[ci] / S.rz_cnt;
+      if (s_step.kind == SK_RZ_LOCAL || s_step.kind == SK_RZ_MERGE || s_step.kind == SK_RZ_FINAL)
+        per_rz = __ldg(L.need + ci) / s_step.rz_cnt;
       for (int k = 0; k < it.count; ++k) {
-        run_subitem(J, S, it.first + k, per_rz, smem_raw, L);
+        run_subitem(it.first + k, per_rz, L);
         __syncthreads();
       }
     }
@@ -288,8 +326,8 @@ __global__ void __launch_bounds__(EXEC_THREADS, 2) k_exec(ExecLaunch L) {
 
 }  // namespace
 
-size_t exec_smem_bytes(int group_buffers, int group_bh, int group_bw) {
-  size_t g = (size_t)group_buffers * group_bh * group_bw * 4;
+size_t exec_smem_bytes(int group_buffers, int group_rows, int tile_words) {
+  size_t g = GROUP_PROG_BYTES + (size_t)group_buffers * group_buffer_bytes(group_rows, tile_words);
   size_t m = sizeof(CclSmem);
   if (sizeof(SelectSmem) > m) m = sizeof(SelectSmem);
   const size_t arith = (size_t)kArithMaxRegs * EXEC_THREADS * 4 + sizeof(ArithInsn) * kArithMaxInsns;

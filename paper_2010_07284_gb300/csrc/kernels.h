@@ -117,14 +117,13 @@ struct ExecLaunch {
   const int32_t* need;     // per (job, step) sub-items in total
   int64_t spin_limit;
   int32_t group_buffers;   // shared-memory buffers per group tile
-  int32_t group_bh;        // rows per buffer (gth + 2*HMAX)
-  int32_t group_bw;        // words per buffer (gtww + 2)
   int32_t grid;            // CTAs
   int32_t smem_bytes;      // dynamic shared memory per CTA (groups stage rank
                            // planes in what their buffers leave free)
   unsigned long long* trace;  // optional: per (job, step) {start, end, busy, wait} in ns
 };
-size_t exec_smem_bytes(int group_buffers, int group_bh, int group_bw);
+// group_rows: rows of a buffer (tile rows + 2 * the largest halo).
+size_t exec_smem_bytes(int group_buffers, int group_rows, int tile_words);
 cudaError_t exec_configure(size_t smem_bytes, int* max_ctas_per_sm);
 cudaError_t launch_exec(const ExecLaunch& L, cudaStream_t st);
 

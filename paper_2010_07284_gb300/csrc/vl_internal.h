@@ -30,9 +30,20 @@ constexpr int CCL_MAXBORDER = 2 * CCL_TWW * 16 + 2 * CCL_TH;
 constexpr int EXEC_THREADS = 512;  // threads per CTA of every tiled kernel
 constexpr int EXEC_WARPS = EXEC_THREADS / 32;
 
-// Shared memory that a context sets aside for the buffers of group tiles (14
-// buffers of a 32 x 32-word tile with 8 halo rows above and below).
-constexpr int kGroupBudget = 14 * 48 * 34 * 4;
+// Buffers of a fused group: rows of 16-byte vectors, the tile's words and one
+// vector left and right of them (vectors per row, bytes of one buffer).
+VL_HD_INLINE int group_vecs(int tile_words) { return (tile_words + 3) / 4 + 2; }
+static inline int64_t group_buffer_bytes(int rows, int tile_words) {
+  return (int64_t)rows * group_vecs(tile_words) * 16;
+}
+// Shared memory in front of the buffers: instructions of a segment (and one
+// behind them), and which of them are loads.
+constexpr int GROUP_SEG = 256;
+constexpr int64_t GROUP_PROG_BYTES = (GROUP_SEG + 1) * 16 + (GROUP_SEG + 8) * 2;
+static_assert(GROUP_PROG_BYTES % 16 == 0, "buffers start on 16-byte boundaries");
+// Shared memory the buffers of a context's largest tiles may take: 14
+// buffers of a 32 x 32-word tile with 8 halo rows above and below.
+constexpr int64_t kGroupBudget = 14 * 48 * 10 * 16;
 
 // Device status word values (match vl_status where they overlap).
 constexpr int ST_OK = 0;
@@ -130,7 +141,8 @@ struct StepDesc {
   int32_t rz_off;    // rho batches: first RZ entry
   int32_t rz_cnt;
   int32_t pct_off;   // percentile step: first PCT entry
-  int32_t pct_cnt;
+  int32_t pct_cnt;   // (groups, on the device: loads in pct_off, float thresholds in
+                     //   pct_cnt among its instructions)
   int32_t rank_mask; // groups: rank tables (< 32) its I_RTHR read, one bit each
   int32_t rank_halo; // groups: largest halo of those I_RTHR
   int32_t n_bufs;    // groups: tile buffers its instructions use (0 .. n_bufs-1);
@@ -196,7 +208,12 @@ struct DevJob {
   int32_t conn;
   int32_t n_images;
   const DevImage* images;
-  uint32_t* const* slots;       // materialised mask slots
+  uint32_t* const* slots;       // materialised mask slots: the intermediate
+                                // ones back to back at slot_mem, the roots'
+                                // at root_mem, then those of mask images
+  uint32_t* slot_mem;
+  uint32_t* root_mem;
+  int32_t n_inter_slots, n_root_slots;
   const Insn* insns;
   const StepDesc* steps;        // this job's formula steps
   const int32_t* dep_off;       // step dependencies (CSR, job-relative steps)
