@@ -157,6 +157,39 @@ int ccl_merge_chunks(int H, int Wp, int cth) {
   return (int)std::max<long long>(1, (n + warps - 1) / warps);
 }
 
+// The steps of a plan as the executor runs them: with split selects, the
+// percentile step follows the passes that many blocks share.
+struct DevSteps {
+  std::vector<StepDesc> steps;
+  std::vector<int32_t> dep_off, deps;
+};
+DevSteps device_steps(const Plan& P, bool split_selects) {
+  DevSteps D;
+  std::vector<int32_t> at(P.steps.size());
+  D.dep_off.push_back(0);
+  for (size_t i = 0; i < P.steps.size(); ++i) {
+    const auto own_deps = [&] {
+      for (int q = P.dep_off[i]; q < P.dep_off[i + 1]; ++q) D.deps.push_back(at[P.deps[q]]);
+    };
+    const bool split = split_selects && P.steps[i].kind == SK_PCT;
+    for (int d = 0; split && d < SEL_PASSES; ++d) {
+      StepDesc h = P.steps[i];
+      h.kind = SK_PCT_PASS;
+      h.halo = d;
+      if (d == 0) own_deps();
+      else D.deps.push_back((int32_t)D.steps.size() - 1);
+      D.dep_off.push_back((int32_t)D.deps.size());
+      D.steps.push_back(h);
+    }
+    if (split) D.deps.push_back((int32_t)D.steps.size() - 1);
+    else own_deps();
+    D.dep_off.push_back((int32_t)D.deps.size());
+    at[i] = (int32_t)D.steps.size();
+    D.steps.push_back(P.steps[i]);
+  }
+  return D;
+}
+
 }  // namespace
 
 // ================================================================ batch ==
@@ -204,10 +237,10 @@ vl_status batch_build(vl_context* ctx, const vl_job* jobs, int n_jobs, cudaStrea
   struct JobInfo {
     const Plan* P;
     int H, W, Wp, pitch;
-    int gty, gtx, cty, ctx_, ctiles, cth;
+    int gty, gtx, cty, ctx_, ctiles, cth, sel_blocks;
     std::vector<int> need;
     size_t off_images, off_slotptrs, off_pct, off_slots, off_rz, set_bytes, set_off[2];
-    size_t off_roots, off_status, off_planes, off_num;
+    size_t off_roots, off_status, off_planes, off_num, off_hist;
     int n_table;  // image table: the formula's images, then its number images
     int step_base;
     int formula_idx;
@@ -237,21 +270,6 @@ vl_status batch_build(vl_context* ctx, const vl_job* jobs, int n_jobs, cudaStrea
   size_t off = 0;
   auto take = [&](size_t bytes, size_t a = 256) { off = align_up(off, a); size_t o = off; off += bytes; return o; };
   const size_t off_jobs = take(sizeof(DevJob) * n_jobs);
-  std::vector<size_t> f_steps(formulas.size()), f_insns(formulas.size()), f_rz(formulas.size()),
-      f_pct(formulas.size()), f_rtab(formulas.size()), f_rvals(formulas.size()),
-      f_doff(formulas.size()), f_deps(formulas.size()), f_arith(formulas.size());
-  for (size_t k = 0; k < formulas.size(); ++k) {
-    const Plan* P = formulas[k];
-    f_steps[k] = take(sizeof(StepDesc) * std::max<size_t>(1, P->steps.size()));
-    f_insns[k] = take(sizeof(Insn) * std::max<size_t>(1, P->insns.size()));
-    f_rz[k] = take(sizeof(RzDesc) * std::max<size_t>(1, P->rz.size()));
-    f_pct[k] = take(sizeof(PctDesc) * std::max<size_t>(1, P->pct.size()));
-    f_rtab[k] = take(sizeof(RankTab) * std::max<size_t>(1, P->rtab.size()));
-    f_rvals[k] = take(sizeof(float) * std::max<size_t>(1, P->rvals.size()));
-    f_doff[k] = take(sizeof(int32_t) * std::max<size_t>(1, P->dep_off.size()));
-    f_deps[k] = take(sizeof(int32_t) * std::max<size_t>(1, P->deps.size()));
-    f_arith[k] = take(sizeof(ArithInsn) * std::max<size_t>(1, P->arith.size()));
-  }
   const TileShape ts = force ? *force : pick_tile_shape(ctx, jobs, n_jobs, nullptr, !persistent);
   if (ts.per_op) {
     if (n_jobs != 1 || persistent)
@@ -260,9 +278,36 @@ vl_status batch_build(vl_context* ctx, const vl_job* jobs, int n_jobs, cudaStrea
   }
   if (!tile_shape_fits(ctx, ts)) return set_err(ctx, VL_ERR_ARG, "tile shape does not fit shared memory");
   const int cps = ts.ctas_per_sm > 0 ? std::min(ts.ctas_per_sm, ctx->ctas_per_sm) : ctx->ctas_per_sm;
+  const int grid = std::max(1, ctx->sm_count * cps);
+  // A percentile select is one block's work when there are as many as blocks,
+  // or the channels are small: five selects of one 256 x 256 image take 30 us
+  // that way and 40 us as passes that many blocks share (five more steps),
+  // of 384 x 384 56 and 48 us, of 512 x 512 about 105 and 44 us.
+  int64_t n_selects = 0, select_px = 0;
+  for (int j = 0; j < n_jobs; ++j) {
+    n_selects += (int64_t)J[j].P->pct.size();
+    if (!J[j].P->pct.empty()) select_px = std::max<int64_t>(select_px, (int64_t)J[j].H * J[j].W);
+  }
+  const bool split_selects = n_selects > 0 && n_selects < grid && select_px >= (1 << 18);
+  std::vector<DevSteps> F;
+  for (const Plan* P : formulas) F.push_back(device_steps(*P, split_selects));
+  std::vector<size_t> f_steps(formulas.size()), f_insns(formulas.size()), f_rz(formulas.size()),
+      f_pct(formulas.size()), f_rtab(formulas.size()), f_rvals(formulas.size()),
+      f_doff(formulas.size()), f_deps(formulas.size()), f_arith(formulas.size());
+  for (size_t k = 0; k < formulas.size(); ++k) {
+    const Plan* P = formulas[k];
+    f_steps[k] = take(sizeof(StepDesc) * std::max<size_t>(1, F[k].steps.size()));
+    f_insns[k] = take(sizeof(Insn) * std::max<size_t>(1, P->insns.size()));
+    f_rz[k] = take(sizeof(RzDesc) * std::max<size_t>(1, P->rz.size()));
+    f_pct[k] = take(sizeof(PctDesc) * std::max<size_t>(1, P->pct.size()));
+    f_rtab[k] = take(sizeof(RankTab) * std::max<size_t>(1, P->rtab.size()));
+    f_rvals[k] = take(sizeof(float) * std::max<size_t>(1, P->rvals.size()));
+    f_doff[k] = take(sizeof(int32_t) * std::max<size_t>(1, F[k].dep_off.size()));
+    f_deps[k] = take(sizeof(int32_t) * std::max<size_t>(1, F[k].deps.size()));
+    f_arith[k] = take(sizeof(ArithInsn) * std::max<size_t>(1, P->arith.size()));
+  }
   int total_steps = 0;
   std::vector<WorkItem> items;
-  const int grid = std::max(1, ctx->sm_count * cps);
   for (int j = 0; j < n_jobs; ++j) {
     JobInfo& I = J[j];
     const Plan& P = *I.P;
@@ -283,11 +328,13 @@ vl_status batch_build(vl_context* ctx, const vl_job* jobs, int n_jobs, cudaStrea
     I.ctx_ = ccl_tiles_x(I.Wp);
     I.ctiles = I.cty * I.ctx_;
     I.step_base = total_steps;
-    total_steps += (int)P.steps.size();
-    for (const StepDesc& s : P.steps) {
+    I.sel_blocks = split_selects ? select_blocks((int64_t)I.H * I.W, n_selects, grid) : 0;
+    total_steps += (int)F[I.formula_idx].steps.size();
+    for (const StepDesc& s : F[I.formula_idx].steps) {
       int n = 1;
       switch (s.kind) {
         case SK_PCT: n = s.pct_cnt; break;
+        case SK_PCT_PASS: n = s.pct_cnt * I.sel_blocks; break;
         case SK_GROUP: n = I.gty * I.gtx; break;
         case SK_RZ_LOCAL: case SK_RZ_FINAL: n = s.rz_cnt * I.ctiles; break;
         case SK_RZ_MERGE:
@@ -325,11 +372,12 @@ vl_status batch_build(vl_context* ctx, const vl_job* jobs, int n_jobs, cudaStrea
     std::vector<SchedJob> sj(n_jobs);
     for (int j = 0; j < n_jobs; ++j) {
       const Plan& P = *J[j].P;
-      sj[j].dep_off = P.dep_off.data();
-      sj[j].deps = P.deps.data();
+      const DevSteps& D = F[J[j].formula_idx];
+      sj[j].dep_off = D.dep_off.data();
+      sj[j].deps = D.deps.data();
       const double tile_scale = (double)ts.rows * ts.words / (16.0 * 32.0);
       for (size_t si = 0; si < J[j].need.size(); ++si) {
-        const StepDesc& sd = P.steps[si];
+        const StepDesc& sd = D.steps[si];
         const int n = J[j].need[si];
         // estimated microseconds per sub-item (one GB300, two CTAs per SM)
         double sub_us;
@@ -347,7 +395,11 @@ vl_status batch_build(vl_context* ctx, const vl_job* jobs, int n_jobs, cudaStrea
           case SK_RZ_FINAL: sub_us = 10.0 * J[j].cth / CCL_TH; break;
           case SK_RANK: sub_us = 50.0; break;
           case SK_ARITH: sub_us = 10.0 + 2.0 * sd.insn_cnt; break;
-          default: sub_us = 100.0; break;
+          // a select by one block: 10 us and 3 pixels a ns; a share of one
+          case SK_PCT_PASS: sub_us = 10.0; break;
+          default:
+            sub_us = J[j].sel_blocks ? 5.0 : 10.0 + (double)J[j].H * J[j].W / 3000.0;
+            break;
         }
         int chunk = std::max(1, (n + 4 * grid - 1) / (4 * grid));
         if (plenty) {
@@ -369,9 +421,12 @@ vl_status batch_build(vl_context* ctx, const vl_job* jobs, int n_jobs, cudaStrea
   const size_t off_items = take(sizeof(WorkItem) * std::max<size_t>(1, items.size()));
   const size_t off_need = take(sizeof(int32_t) * std::max(1, total_steps));
   // counters: head, done[steps] -- zeroed before every run
+  // (and the state of selects that many blocks share)
   const size_t off_counters = take(sizeof(int32_t) * (1 + total_steps));
-  const size_t counters_bytes = sizeof(int32_t) * (1 + total_steps);
   const size_t tables_end = off;
+  for (int j = 0; j < n_jobs; ++j)
+    J[j].off_hist = split_selects ? take(sizeof(uint32_t) * SEL_HIST * J[j].P->pct.size()) : 0;
+  const size_t counters_bytes = off - off_counters;
   // buffers
   for (int j = 0; j < n_jobs; ++j) {
     JobInfo& I = J[j];
@@ -420,10 +475,11 @@ vl_status batch_build(vl_context* ctx, const vl_job* jobs, int n_jobs, cudaStrea
   std::vector<char> host(tables_end, 0);
   for (size_t k = 0; k < formulas.size(); ++k) {
     const Plan* P = formulas[k];
-    if (!P->steps.empty()) std::memcpy(&host[f_steps[k]], P->steps.data(), sizeof(StepDesc) * P->steps.size());
+    const DevSteps& D = F[k];
+    if (!D.steps.empty()) std::memcpy(&host[f_steps[k]], D.steps.data(), sizeof(StepDesc) * D.steps.size());
     // on the device a group's pct_cnt counts its float thresholds, pct_off its loads
     StepDesc* hs = reinterpret_cast<StepDesc*>(&host[f_steps[k]]);
-    for (size_t q = 0; q < P->steps.size(); ++q)
+    for (size_t q = 0; q < D.steps.size(); ++q)
       for (int i = 0; hs[q].kind == SK_GROUP && i < hs[q].insn_cnt; ++i) {
         const int op = insn_op(P->insns[hs[q].insn_off + i]);
         hs[q].pct_cnt += op == I_THR;
@@ -434,8 +490,8 @@ vl_status batch_build(vl_context* ctx, const vl_job* jobs, int n_jobs, cudaStrea
     if (!P->pct.empty()) std::memcpy(&host[f_pct[k]], P->pct.data(), sizeof(PctDesc) * P->pct.size());
     if (!P->rtab.empty()) std::memcpy(&host[f_rtab[k]], P->rtab.data(), sizeof(RankTab) * P->rtab.size());
     if (!P->rvals.empty()) std::memcpy(&host[f_rvals[k]], P->rvals.data(), sizeof(float) * P->rvals.size());
-    if (!P->dep_off.empty()) std::memcpy(&host[f_doff[k]], P->dep_off.data(), sizeof(int32_t) * P->dep_off.size());
-    if (!P->deps.empty()) std::memcpy(&host[f_deps[k]], P->deps.data(), sizeof(int32_t) * P->deps.size());
+    if (!D.dep_off.empty()) std::memcpy(&host[f_doff[k]], D.dep_off.data(), sizeof(int32_t) * D.dep_off.size());
+    if (!D.deps.empty()) std::memcpy(&host[f_deps[k]], D.deps.data(), sizeof(int32_t) * D.deps.size());
     if (!P->arith.empty()) std::memcpy(&host[f_arith[k]], P->arith.data(), sizeof(ArithInsn) * P->arith.size());
   }
   DevJob* hj = reinterpret_cast<DevJob*>(&host[off_jobs]);
@@ -447,7 +503,7 @@ vl_status batch_build(vl_context* ctx, const vl_job* jobs, int n_jobs, cudaStrea
     const Plan& P = *I.P;
     DevJob d{};
     d.H = I.H; d.W = I.W; d.Wp = I.Wp; d.pitch = I.pitch;
-    d.n_steps = (int)P.steps.size();
+    d.n_steps = (int)F[I.formula_idx].steps.size();
     d.step_base = I.step_base;
     d.gth = ts.rows; d.gtww = ts.words;
     d.g_tiles_y = I.gty; d.g_tiles_x = I.gtx;
@@ -488,6 +544,8 @@ vl_status batch_build(vl_context* ctx, const vl_job* jobs, int n_jobs, cudaStrea
     d.rz = reinterpret_cast<const RzDesc*>(tb + f_rz[k]);
     d.pct = reinterpret_cast<const PctDesc*>(tb + f_pct[k]);
     d.pct_val = reinterpret_cast<float*>(tb + I.off_pct);
+    d.sel_hist = split_selects && !P.pct.empty() ? reinterpret_cast<uint32_t*>(tb + I.off_hist) : nullptr;
+    d.sel_blocks = I.sel_blocks;
     d.rtab = reinterpret_cast<const RankTab*>(tb + f_rtab[k]);
     d.rvals = reinterpret_cast<const float*>(tb + f_rvals[k]);
     d.n_rtab = (int32_t)P.rtab.size();
@@ -527,10 +585,10 @@ vl_status batch_build(vl_context* ctx, const vl_job* jobs, int n_jobs, cudaStrea
     if (e) return cuda_err(ctx, e, "allocating the step timeline");
     L.trace = static_cast<unsigned long long*>(b->trace->ptr);
     for (int j = 0; j < n_jobs; ++j)
-      for (size_t s2 = 0; s2 < J[j].P->steps.size(); ++s2) {
+      for (size_t s2 = 0; s2 < F[J[j].formula_idx].steps.size(); ++s2) {
         b->trace_meta.push_back(j);
         b->trace_meta.push_back((int32_t)s2);
-        b->trace_meta.push_back(J[j].P->steps[s2].kind);
+        b->trace_meta.push_back(F[J[j].formula_idx].steps[s2].kind);
       }
   }
   // ---- results
@@ -790,19 +848,16 @@ vl_status plain_enqueue(vl_context* ctx, const Plan& P, vl_image* const* imgs, i
   DevBlockPtr pct, sel_scratch;
   if (P.n_pct_slots) {
     if ((e = dev_alloc(ctx, sizeof(float) * P.n_pct_slots, st, &pct))) return cuda_err(ctx, e, "allocating percentiles");
-    // channels of a million pixels and more take the grid-wide select
-    const bool wide = (long long)H * W >= (1LL << 20);
-    if (wide && (e = dev_alloc(ctx, select_wide_scratch_bytes(), st, &sel_scratch)))
+    if ((e = dev_alloc(ctx, select_scratch_bytes((int)P.pct.size()), st, &sel_scratch)))
       return cuda_err(ctx, e, "allocating select scratch");
+    std::vector<SelJob> sel;
     for (const PctDesc& d : P.pct) {
-      const long long n = (long long)H * W;
-      const long long rank = (long long)(d.q * (double)(n - 1));
       const Chan c = chan(d.img, d.ch);
-      float* o = static_cast<float*>(pct->ptr) + d.slot;
-      e = wide ? launch_select_wide(c.p, c.format, pitch, H, W, rank, o, sel_scratch->ptr, st)
-               : launch_select(c.p, c.format, pitch, H, W, rank, o, st);
-      if (e) return cuda_err(ctx, e, "launching a percentile select");
+      sel.push_back(SelJob{c.p, c.format, (long long)(d.q * (double)((long long)H * W - 1)),
+                           static_cast<float*>(pct->ptr) + d.slot});
     }
+    if ((e = launch_selects(sel.data(), (int)sel.size(), H, W, pitch, sel_scratch->ptr, st)))
+      return cuda_err(ctx, e, "launching the percentile selects");
   }
   // rho scratch
   DevBlockPtr scratch;

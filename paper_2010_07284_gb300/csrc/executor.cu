@@ -158,17 +158,30 @@ static_assert(sizeof(DevJob) % 8 == 0 && sizeof(StepDesc) <= 128, "copied by one
 // then do not depend on what the others keep alive (inlined into one kernel
 // at 64 registers a thread, the interpreter's loop spilled).
 
-__device__ __noinline__ void percentile_item(int sub) {
-  const DevJob& J = s_job;
-  const StepDesc& S = s_step;
-  SelectSmem& s = *reinterpret_cast<SelectSmem*>(exec_smem);
-  const PctDesc d = J.pct[S.pct_off + sub];
+VL_DEV SelChan select_chan(const DevJob& J, const PctDesc& d) {
   const DevImage im = J.images[d.img];
-  const long long n = (long long)J.H * J.W;
-  const long long rank = (long long)(d.q * (double)(n - 1));
-  const float v = select_rank(s, chan_ptr(im, d.ch, (size_t)J.H * J.pitch), im.format, !im.written,
-                              J.H, J.W, J.pitch, rank);
+  return SelChan{chan_ptr(im, d.ch, (size_t)J.H * J.pitch), im.format, !im.written, J.H, J.W, J.pitch};
+}
+VL_DEV long long select_rank_of(const DevJob& J, const PctDesc& d) {
+  return (long long)(d.q * (double)((long long)J.H * J.W - 1));
+}
+__device__ __noinline__ void percentile_item(int sub, int smem_bytes) {
+  const DevJob& J = s_job;
+  SelectSmem& s = *reinterpret_cast<SelectSmem*>(exec_smem);
+  const PctDesc d = J.pct[s_step.pct_off + sub];
+  const SelChan c = select_chan(J, d);
+  const float v =
+      J.sel_hist ? sel_finish(s, J.sel_hist + (size_t)sub * SEL_HIST, c, select_rank_of(J, d))
+                 : select_rank(s, reinterpret_cast<uint32_t*>(exec_smem + sizeof(SelectSmem)),
+                               (smem_bytes - (int)sizeof(SelectSmem)) / 4, c, select_rank_of(J, d));
   if (threadIdx.x == 0) J.pct_val[d.slot] = v;
+}
+__device__ __noinline__ void percentile_pass_item(int sub) {
+  const DevJob& J = s_job;
+  const int k = sub / J.sel_blocks, block = sub - k * J.sel_blocks;
+  const PctDesc d = J.pct[s_step.pct_off + k];
+  sel_pass(*reinterpret_cast<SelectSmem*>(exec_smem), select_chan(J, d), s_step.halo, block,
+           J.sel_blocks, select_rank_of(J, d), J.sel_hist + (size_t)k * SEL_HIST);
 }
 
 __device__ __noinline__ void group_item(int sub, const ExecLaunch& L) {
@@ -241,7 +254,8 @@ __device__ __noinline__ void rz_merge_item(int sub, int per_rz) {
 
 VL_DEV void run_subitem(int sub, int per_rz, const ExecLaunch& L) {
   switch (s_step.kind) {
-    case SK_PCT: percentile_item(sub); break;
+    case SK_PCT: percentile_item(sub, L.smem_bytes); break;
+    case SK_PCT_PASS: percentile_pass_item(sub); break;
     case SK_GROUP: group_item(sub, L); break;
     case SK_RANK: rank_item(sub); break;
     case SK_ARITH: arith_item(sub); break;

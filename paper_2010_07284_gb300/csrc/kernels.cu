@@ -106,109 +106,27 @@ __global__ void k_near(const uint32_t* __restrict__ a, MaskGeom g, int conn,
 
 // --------------------------------------------------------------- select --
 
-__global__ void __launch_bounds__(EXEC_THREADS) k_select(const void* plane, int format, int pitch,
-                                                         int H, int W, long long rank, float* out) {
-  __shared__ SelectSmem s;
-  float v = select_rank(s, plane, format, true, H, W, pitch, rank);
-  if (threadIdx.x == 0) *out = v;
-}
-
-// Grid-wide radix select for large channels (a volume's 9 M voxels would
-// keep the one-CTA select on a single SM for milliseconds): the same digits
-// (8, 12, 12 bits of the order-preserving key), each pass one histogram
-// kernel over the whole grid (shared-memory bins, then global atomics) and
-// one warp that finds the digit holding the rank.
-struct WideSel {
-  uint32_t prefix, pmask;
-  unsigned long long rank;
+// Percentile selects, many blocks each: block (x, y) takes its share of pass
+// `pass` of select y; then one block per select.
+constexpr int SEL_BATCH = 24;
+struct SelBatch {
+  SelJob job[SEL_BATCH];
+  uint32_t* state;
+  int H, W, pitch;
 };
-
-__global__ void k_sel_init(WideSel* st, long long rank) {
-  st->prefix = 0;
-  st->pmask = 0;
-  st->rank = (unsigned long long)rank;
+__global__ void __launch_bounds__(EXEC_THREADS, 2)
+k_sel_pass(const __grid_constant__ SelBatch B, int pass) {
+  __shared__ __align__(16) SelectSmem s;
+  const SelJob j = B.job[blockIdx.y];
+  sel_pass(s, SelChan{j.plane, j.format, 1, B.H, B.W, B.pitch}, pass, blockIdx.x, gridDim.x, j.rank,
+           B.state + (size_t)blockIdx.y * SEL_HIST);
 }
-
-// Each thread takes SEL_UNR elements a grid stride apart per iteration (their
-// loads in flight together); the row and column of an element are stepped
-// by the stride instead of divided out.  A warp whose elements all fall in
-// one bin (a background value) counts them with one shared atomic, else
-// each element with its own; a warp none of whose elements passes the
-// prefix skips both.
-constexpr int SEL_UNR = 4;
-__global__ void __launch_bounds__(256) k_sel_hist(const void* plane, int format, int pitch, int H,
-                                                  int W, const WideSel* st, int sh, int nb,
-                                                  uint32_t* hist) {
-  __shared__ uint32_t h[4096];
-  for (int i = threadIdx.x; i < nb; i += blockDim.x) h[i] = 0;
-  __syncthreads();
-  const uint32_t prefix = st->prefix, pmask = st->pmask;
-  const int lane = threadIdx.x & 31;
-  const long long n = (long long)H * W;
-  const long long stride = (long long)gridDim.x * blockDim.x;
-  const int sy = (int)(stride / W), sx = (int)(stride - (long long)sy * W);
-  long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  int y = (int)(i / W), x = (int)(i - (long long)y * W);
-  // warp-uniform loop (every lane runs the ballots and the match)
-  for (long long base = (long long)blockIdx.x * blockDim.x; base < n; base += SEL_UNR * stride) {
-    uint32_t key[SEL_UNR];
-    bool in[SEL_UNR];
-#pragma unroll
-    for (int u = 0; u < SEL_UNR; ++u) {
-      in[u] = i < n;
-      key[u] = in[u] ? f2key(ld_px(plane, format, true, (size_t)y * pitch + x)) : 0u;
-      i += stride;
-      y += sy;
-      x += sx;
-      if (x >= W) { x -= W; ++y; }
-    }
-#pragma unroll
-    for (int u = 0; u < SEL_UNR; ++u) {
-      const bool ok = in[u] && (key[u] & pmask) == prefix;
-      if (!__any_sync(0xFFFFFFFFu, ok)) continue;
-      const uint32_t bin = (key[u] >> sh) & (uint32_t)(nb - 1);
-      int same = 0;
-      __match_all_sync(0xFFFFFFFFu, ok ? bin : 0xFFFFFFFFu, &same);
-      if (same) {  // the whole warp in one bin (a background value)
-        if (lane == 0) atomicAdd(&h[bin], 32u);
-      } else if (ok) {
-        atomicAdd(&h[bin], 1u);
-      }
-    }
-  }
-  __syncthreads();
-  for (int i = threadIdx.x; i < nb; i += blockDim.x)
-    if (h[i]) atomicAdd(&hist[i], h[i]);
-}
-
-// One warp: lane l sums bins [l * per, (l + 1) * per); a scan finds the lane
-// whose bins hold the rank, which walks them.  The last pass writes the value.
-__global__ void k_sel_pick(const uint32_t* hist, int sh, int nb, WideSel* st, float* out) {
-  const int lane = threadIdx.x;
-  const int per = nb / 32;
-  unsigned long long sum = 0;
-  for (int q = 0; q < per; ++q) sum += hist[lane * per + q];
-  unsigned long long incl = sum;
-  for (int o = 1; o < 32; o <<= 1) {
-    const unsigned long long t = __shfl_up_sync(FULL, incl, o);
-    if (lane >= o) incl += t;
-  }
-  const unsigned long long rank = st->rank, excl = incl - sum;
-  __syncwarp();
-  if (sum > 0 && excl <= rank && rank < incl) {  // exactly one lane
-    unsigned long long acc = excl;
-    for (int q = 0; q < per; ++q) {
-      const int b = lane * per + q;
-      if (acc + hist[b] > rank) {
-        st->prefix |= (uint32_t)b << sh;
-        st->pmask |= (uint32_t)(nb - 1) << sh;
-        st->rank = rank - acc;
-        if (out) *out = key2f(st->prefix);
-        break;
-      }
-      acc += hist[b];
-    }
-  }
+__global__ void __launch_bounds__(EXEC_THREADS) k_sel_finish(const __grid_constant__ SelBatch B) {
+  __shared__ __align__(16) SelectSmem s;
+  const SelJob j = B.job[blockIdx.x];
+  const float v = sel_finish(s, B.state + (size_t)blockIdx.x * SEL_HIST,
+                             SelChan{j.plane, j.format, 1, B.H, B.W, B.pitch}, j.rank);
+  if (threadIdx.x == 0) *j.out = v;
 }
 
 // ----------------------------------------------------------- arithmetic --
@@ -371,29 +289,33 @@ cudaError_t launch_near(const uint32_t* a, MaskGeom g, int conn, uint32_t* out,
   k_near<<<grid_for((long long)g.H * g.Wp, kThreads * 2), kThreads, 0, st>>>(a, g, conn, out);
   return cudaGetLastError();
 }
-cudaError_t launch_select(const void* plane, int format, int pitch, int H, int W, long long rank,
-                          float* out, cudaStream_t st) {
-  k_select<<<1, EXEC_THREADS, 0, st>>>(plane, format, pitch, H, W, rank, out);
-  return cudaGetLastError();
+size_t select_scratch_bytes(int n) {
+  return (size_t)std::min(n, SEL_BATCH) * SEL_HIST * sizeof(uint32_t);
 }
 
-size_t select_wide_scratch_bytes() { return 4096 * sizeof(uint32_t) + 256; }
-
-cudaError_t launch_select_wide(const void* plane, int format, int pitch, int H, int W,
-                               long long rank, float* out, void* scratch, cudaStream_t st) {
-  uint32_t* hist = static_cast<uint32_t*>(scratch);
-  WideSel* ws = reinterpret_cast<WideSel*>(static_cast<char*>(scratch) + 4096 * sizeof(uint32_t));
-  k_sel_init<<<1, 1, 0, st>>>(ws, rank);
-  cudaError_t e = cudaGetLastError();
-  if (e) return e;
-  const int shifts[3] = {24, 12, 0}, widths[3] = {8, 12, 12};
-  for (int pass = 0; pass < 3; ++pass) {
-    const int nb = 1 << widths[pass];
-    if ((e = cudaMemsetAsync(hist, 0, nb * sizeof(uint32_t), st))) return e;
-    k_sel_hist<<<grid_for((long long)H * W, 256 * 8), 256, 0, st>>>(plane, format, pitch, H, W, ws,
-                                                                   shifts[pass], nb, hist);
-    if ((e = cudaGetLastError())) return e;
-    k_sel_pick<<<1, 32, 0, st>>>(hist, shifts[pass], nb, ws, pass == 2 ? out : nullptr);
+cudaError_t launch_selects(const SelJob* jobs, int n, int H, int W, int pitch, void* scratch,
+                           cudaStream_t st) {
+  for (int at = 0; at < n; at += SEL_BATCH) {
+    SelBatch B{};
+    const int m = std::min(n - at, SEL_BATCH);
+    bool wide = false;
+    for (int i = 0; i < m; ++i) {
+      B.job[i] = jobs[at + i];
+      wide |= B.job[i].format != PX_U16;
+    }
+    B.state = static_cast<uint32_t*>(scratch);
+    B.H = H;
+    B.W = W;
+    B.pitch = pitch;
+    cudaError_t e = cudaMemsetAsync(scratch, 0, select_scratch_bytes(m), st);
+    if (e) return e;
+    const dim3 grid(select_blocks((int64_t)H * W, m, 2 * 152), m);
+    // (16-bit keys: two passes of 12 bits after one that missed)
+    for (int pass = 0; pass < (wide ? SEL_PASSES : 3); ++pass) {
+      k_sel_pass<<<grid, EXEC_THREADS, 0, st>>>(B, pass);
+      if ((e = cudaGetLastError())) return e;
+    }
+    k_sel_finish<<<m, EXEC_THREADS, 0, st>>>(B);
     if ((e = cudaGetLastError())) return e;
   }
   return cudaSuccess;

@@ -31,13 +31,18 @@ cudaError_t launch_andnot(const uint32_t* a, const uint32_t* b, MaskGeom g, uint
 cudaError_t launch_const(MaskGeom g, bool value, uint32_t* out, cudaStream_t st);
 cudaError_t launch_near(const uint32_t* a, MaskGeom g, int conn, uint32_t* out,
                         cudaStream_t st);
-cudaError_t launch_select(const void* plane, int format, int pitch, int H, int W, long long rank,
-                          float* out, cudaStream_t st);
-// The same over the whole grid, for large channels; scratch: device memory
-// of select_wide_scratch_bytes() (reused call after call on one stream).
-size_t select_wide_scratch_bytes();
-cudaError_t launch_select_wide(const void* plane, int format, int pitch, int H, int W,
-                               long long rank, float* out, void* scratch, cudaStream_t st);
+// Percentile selects: the value of rank `rank` of a channel goes to *out.
+// scratch: device memory of select_scratch_bytes(n) (reused call after call
+// on one stream).
+struct SelJob {
+  const void* plane;
+  int format;
+  long long rank;
+  float* out;
+};
+size_t select_scratch_bytes(int n);
+cudaError_t launch_selects(const SelJob* jobs, int n, int H, int W, int pitch, void* scratch,
+                           cudaStream_t st);
 // out = a (op) b per pixel (op an ArithOp, A_ADD .. A_DIV); b null: the
 // constant c.
 cudaError_t launch_arith(int op, const void* a, int a_format, const void* b, int b_format, float c,

@@ -56,6 +56,7 @@ int64_t estimate_bytes(const Plan& P, int H, int W) {
   size_t b = align256(mask * (P.n_inter_slots + P.n_root_slots));
   b += (size_t)P.n_scratch_sets *
        (align256(2 * px * 4) + align256(tstate * 4) + align256(tstate));
+  b += align256(sizeof(uint32_t) * SEL_HIST * P.pct.size());
   b += align256(sizeof(Insn) * P.insns.size()) + align256(sizeof(StepDesc) * P.steps.size()) +
        64 * 1024;
   return (int64_t)b;

@@ -109,6 +109,9 @@ enum StepKind : int32_t {
   SK_RZ_FINAL = 5,   // rho batch, relabel + write Z: item = (rz, tile)
   SK_RANK = 6,       // rank codes of threshold tables: item = (table, row block)
   SK_ARITH = 7,      // number terms: item = row block, writes the number images
+  SK_PCT_PASS = 8,   // (on the device only: a pass of percentile selects,
+                     //   item = (percentile slot, share of the channel); which
+                     //   pass in `halo`)
 };
 
 // Rows of one arithmetic work item.
@@ -132,6 +135,20 @@ static_assert(sizeof(ArithInsn) == 12, "ArithInsn layout");
 
 // Rows of one rank-code work item.
 constexpr int RANK_ROWS = 8;
+
+// Percentile selects over many blocks: passes (one on the range a sample
+// gives; three more, of 12 bits each, if that misses), words of a select in
+// global memory, and how many blocks share a select when `side_by_side`
+// selects run at once on `slots` resident blocks: enough to fill those,
+// each with at least 8192 pixels (one round of its threads' loads).
+constexpr int SEL_PASSES = 4;
+constexpr int SEL_BINS = 4096;
+constexpr int SEL_HIST = 16 + SEL_PASSES * SEL_BINS;
+static inline int select_blocks(int64_t pixels, int64_t side_by_side, int64_t slots) {
+  int64_t n = slots / side_by_side, most = (pixels + 8191) / 8192;
+  if (n > most) n = most;
+  return n < 1 ? 1 : (int)n;
+}
 
 struct StepDesc {
   int32_t kind;
@@ -221,6 +238,8 @@ struct DevJob {
   const RzDesc* rz;
   const PctDesc* pct;
   float* pct_val;               // percentile values by slot
+  uint32_t* sel_hist;           // state of the percentile selects (SEL_HIST words
+                                //   each), null: a select is one block's work
   // CCL scratch sets, one per select of a batch step, `set_bytes` apart:
   // union-find over keys (G, 2 * H * W entries: pixel ids and the keys of
   // unseeded components), saved tile state (tiles x tile_cap words)
@@ -233,7 +252,7 @@ struct DevJob {
   const RankTab* rtab;          // rank tables of the formula
   const float* rvals;           //   their sorted threshold values
   int32_t n_rtab;
-  int32_t pad_;
+  int32_t sel_blocks;           // blocks that share a percentile select
   uint32_t* planes;             // rank-code planes, H x Wp words each
   const ArithInsn* arith;       // number-term program (SK_ARITH)
   int32_t n_arith;
