@@ -864,13 +864,13 @@ vl_status plain_enqueue(vl_context* ctx, const Plan& P, vl_image* const* imgs, i
   CclScratch sc{};
   Rz3Scratch sc3{};
   if (!P.rz.empty() && vol) {
-    // labels of phi2, a flag per component, the seed voxels, tile state
+    // union-find of phi2, a flag per component, tile state
     const size_t px = (size_t)H * W;
     const size_t tiles = (size_t)ccl_tiles_y(H, g.Hs) * ccl_tiles_x(Wp);
     const int tcap = ccl_tile_cap_host(Wp);
     size_t off = 0;
     auto take = [&](size_t b) { off = align_up(off, 256); size_t o = off; off += b; return o; };
-    const size_t oL = take(px * 4), oF = take(px), oS = take(mask_bytes), oP = take(tiles * tcap * 4),
+    const size_t oL = take(px * 4), oF = take(px), oP = take(tiles * tcap * 4),
                  oT = take(tiles * tcap);
     if ((e = dev_alloc(ctx, align_up(off, 256), st, &scratch)))
       return cuda_err(ctx, e, "allocating select scratch");
@@ -880,7 +880,6 @@ vl_status plain_enqueue(vl_context* ctx, const Plan& P, vl_image* const* imgs, i
     sc3.ccl.tpar = reinterpret_cast<int32_t*>(p + oP);
     sc3.ccl.tflag = reinterpret_cast<uint8_t*>(p + oT);
     sc3.F = reinterpret_cast<uint8_t*>(p + oF);
-    sc3.seed = reinterpret_cast<uint32_t*>(p + oS);
   } else if (!P.rz.empty()) {
     const size_t px = (size_t)H * W;
     const size_t tiles = (size_t)ccl_tiles_y(H, 0, ccl_rows(g)) * ccl_tiles_x(Wp);

@@ -93,7 +93,6 @@ cudaError_t launch_labels3(const uint32_t* mask, MaskGeom g, int conn, CclScratc
 struct Rz3Scratch {
   CclScratch ccl;   // G: H*W int32 labels of phi2
   uint8_t* F;       // H*W bytes: flag per component root
-  uint32_t* seed;   // H x Wp words
 };
 cudaError_t launch_rz3(const uint32_t* phi1, const uint32_t* phi2, MaskGeom g, int conn,
                        Rz3Scratch sc, uint32_t* Z, int32_t* status, cudaStream_t st);

@@ -14,8 +14,8 @@
 //          (z + 1, y) voxel on voxel (6); then every voxel takes its root.
 //          Labels are canonical: the minimum linear index z*H*W + y*W + x.
 //   rho -- as for images (Sec. 3.2): rho phi1[phi2] = N(phi1 or Z), Z the
-//          phi2-components that meet N phi1; Z from the full labels of phi2,
-//          a flag per component root set from the seed voxels.
+//          phi2-components that meet N phi1; Z from the phi2-components' union-find,
+//          a flag per root set from the seed voxels.
 #include "dev_ccl.cuh"
 #include "dev_common.cuh"
 #include "kernels.h"
@@ -38,66 +38,140 @@ VL_DEV uint32_t word_at(const uint32_t* a, int Wp, int row, int w) {
   return (w >= 0 && w < Wp) ? __ldg(a + (size_t)row * Wp + w) : 0u;
 }
 
-// out = N a, or (N a) and `with` when `with` is given.
-__global__ void k_near3(const uint32_t* __restrict__ a, MaskGeom g, int conn,
-                        const uint32_t* __restrict__ with, uint32_t* __restrict__ out) {
+// N a on word w of row y of the stored image.
+VL_DEV uint32_t near3_word(const uint32_t* a, const MaskGeom& g, int conn, int y, int w) {
   const int Hs = slice_rows(g), D = g.H / Hs;
+  const int z = y / Hs, yz = y - z * Hs;
+  uint32_t res;
+  if (conn == 26) {
+    uint32_t l = 0, c = 0, r = 0;  // OR of the 9 rows around, per column word
+#pragma unroll
+    for (int dz = -1; dz <= 1; ++dz)
+#pragma unroll
+      for (int dy = -1; dy <= 1; ++dy) {
+        if (z + dz < 0 || z + dz >= D || yz + dy < 0 || yz + dy >= Hs) continue;
+        const int row = y + dz * Hs + dy;
+        l |= word_at(a, g.Wp, row, w - 1);
+        c |= word_at(a, g.Wp, row, w);
+        r |= word_at(a, g.Wp, row, w + 1);
+      }
+    res = hdil(l, c, r);
+  } else {
+    res = hdil(word_at(a, g.Wp, y, w - 1), word_at(a, g.Wp, y, w), word_at(a, g.Wp, y, w + 1));
+    if (yz > 0) res |= word_at(a, g.Wp, y - 1, w);
+    if (yz + 1 < Hs) res |= word_at(a, g.Wp, y + 1, w);
+    if (z > 0) res |= word_at(a, g.Wp, y - Hs, w);
+    if (z + 1 < D) res |= word_at(a, g.Wp, y + Hs, w);
+  }
+  return res & vmask(w, g.W);
+}
+
+__global__ void k_near3(const uint32_t* __restrict__ a, MaskGeom g, int conn,
+                        uint32_t* __restrict__ out) {
   const long long nwords = (long long)g.H * g.Wp;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < nwords;
        i += (long long)gridDim.x * blockDim.x) {
     int y, w;
     split_index(i, g.Wp, y, w);
-    const int z = y / Hs, yz = y - z * Hs;
-    uint32_t res;
-    if (conn == 26) {
-      uint32_t l = 0, c = 0, r = 0;  // OR of the 9 rows around, per column word
-      for (int dz = -1; dz <= 1; ++dz) {
-        const int zz = z + dz;
-        if (zz < 0 || zz >= D) continue;
-        for (int dy = -1; dy <= 1; ++dy) {
-          const int yy = yz + dy;
-          if (yy < 0 || yy >= Hs) continue;
-          const int row = zz * Hs + yy;
-          l |= word_at(a, g.Wp, row, w - 1);
-          c |= word_at(a, g.Wp, row, w);
-          r |= word_at(a, g.Wp, row, w + 1);
-        }
-      }
-      res = hdil(l, c, r);
-    } else {
-      res = hdil(word_at(a, g.Wp, y, w - 1), word_at(a, g.Wp, y, w), word_at(a, g.Wp, y, w + 1));
-      if (yz > 0) res |= word_at(a, g.Wp, y - 1, w);
-      if (yz + 1 < Hs) res |= word_at(a, g.Wp, y + 1, w);
-      if (z > 0) res |= word_at(a, g.Wp, y - Hs, w);
-      if (z + 1 < D) res |= word_at(a, g.Wp, y + Hs, w);
-    }
-    res &= vmask(w, g.W);
-    if (with) res &= __ldg(with + i);
-    out[i] = res;
+    out[i] = near3_word(a, g, conn, y, w);
   }
 }
 
-// Unite the components of slices z and z + 1: one warp per row pair (z, y)
-// -- placed by a 32-bit division -- looping over the row's words and, for
-// 26-adjacency, the rows y - 1, y, y + 1 of slice z + 1.
-// L holds, for every voxel of the mask, its component's key (after the 2D
-// pass: the minimum index of its slice component, which is a root).
+// Word w of row yz of slice z, without padding; 0 outside the volume.
+struct SliceRows {
+  const uint32_t* m;
+  int W, Wp, Hs, w;
+  uint32_t edge[3];  // pixels of words w - 1, w, w + 1 inside the image
+  VL_DEV SliceRows(const uint32_t* m_, const MaskGeom& g, int w_)
+      : m(m_), W(g.W), Wp(g.Wp), Hs(slice_rows(g)), w(w_) {
+    edge[0] = w > 0 ? FULL : 0u;
+    edge[1] = vmask(w, W);
+    edge[2] = w + 1 < Wp ? vmask(w + 1, W) : 0u;
+  }
+  VL_DEV uint32_t at(int z, int yz, int d) const {
+    return yz >= 0 && yz < Hs && edge[d + 1]
+               ? __ldg(m + (size_t)(z * Hs + yz) * Wp + w + d) & edge[d + 1] : 0u;
+  }
+};
+
+// Bits of `hit` spread down through the runs of c they lie in.
+VL_DEV uint32_t fill_down(uint32_t hit, uint32_t c) {
+  uint32_t t = hit & c, p = c;
+#pragma unroll
+  for (int o = 1; o < 32; o *= 2) {
+    t |= p & (t >> o);
+    p &= p >> o;
+  }
+  return t;
+}
+
+// Unite the components of slices z and z + 1; one thread per word of slice z.
+// L holds, for every voxel of the mask, its slice component's key (after the
+// 2D pass: the component's minimum index, which is a root).
+//
+// What costs is the unions, each a chain of dependent loads, so the voxel
+// pairs (p, q) across the slices are thinned out with bit operations until
+// one or two per contact remain.  Straight pairs (p over q): of every run of
+// contacts in a row one is taken, and none when the run touches a contact of
+// the row above (p and q are then connected inside their slices to a pair
+// taken there).  Pairs of neighbours that are not straight (26-adjacency)
+// count only where neither voxel has a straight contact (else q, or p, is a
+// slice neighbour of that contact); one row apart, diagonal ones only where
+// the voxel beside p in its row and the one beside q in its own are clear
+// (else that one makes a pair one column closer), and of neighbouring pairs
+// in the same direction the first.  (A warp per row that offered every run
+// start of either row took 147 to 284 us on a 155 x 240 x 240 scan; this
+// takes 50 to 104.)
 __global__ void k_zmerge(const uint32_t* m, MaskGeom g, int conn, int32_t* L, int32_t* status) {
   const int Hs = slice_rows(g), D = g.H / Hs;
-  const int nd = conn == 26 ? 3 : 1;
-  const long long rows = (long long)(D - 1) * Hs;
   const int npx = g.H * g.W;
-  const long long wpb = blockDim.x >> 5;
-  for (long long r = blockIdx.x * wpb + (threadIdx.x >> 5); r < rows; r += gridDim.x * wpb) {
-    int z, yz;  // uniform across the warp
-    split_index(r, Hs, z, yz);
-    for (int w = 0; w < g.Wp; ++w)
-      for (int k = 0; k < nd; ++k) {
-        const int yb = yz + (nd == 3 ? k - 1 : 0);
-        if (yb < 0 || yb >= Hs) continue;
-        ccl_merge_rows(m, g.W, g.Wp, z * Hs + yz, (z + 1) * Hs + yb, w, conn == 26 ? 8 : 4, L,
-                       npx, status);
+  const long long n = (long long)(D - 1) * Hs * g.Wp;
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+       i += (long long)gridDim.x * blockDim.x) {
+    int row, w, z, yz;
+    split_index(i, g.Wp, row, w);
+    split_index(row, Hs, z, yz);
+    const SliceRows R(m, g, w);
+    const uint32_t a = R.at(z, yz, 0);
+    if (!a) continue;
+    const int p0 = row * g.W + 32 * w, q0 = p0 + Hs * g.W;  // first voxels of the words
+    auto unite = [&](uint32_t set, int dq) {
+      while (set) {
+        const int b = __ffs(set) - 1;
+        set &= set - 1;
+        const int ka = ldcg(&L[p0 + b]), kb = ldcg(&L[q0 + b + dq]);
+        if (ka != kb) g_union(L, ka, kb, npx, status);
       }
+    };
+    const uint32_t b0 = R.at(z + 1, yz, 0), c = a & b0;
+    const uint32_t al = R.at(z, yz, -1), bl = R.at(z + 1, yz, -1);
+    const uint32_t au = R.at(z, yz - 1, 0), bu = R.at(z + 1, yz - 1, 0);
+    uint32_t cu = au & bu;  // contacts of the row above
+    if (conn == 26) cu |= (cu << 1) | (cu >> 1);
+    const uint32_t starts = c & ~((c << 1) | ((al & bl) >> 31));
+    unite(starts & ~fill_down(cu, c), 0);
+    if (conn != 26) continue;
+    const uint32_t p = a & ~b0;
+    if (!p) continue;
+    const uint32_t ar = R.at(z, yz, 1), br = R.at(z + 1, yz, 1);
+    // same row, one column apart
+    const uint32_t q = b0 & ~a;
+    unite(p & ((q << 1) | ((bl & ~al) >> 31)), -1);
+    unite(p & ((q >> 1) | ((br & ~ar) << 31)), 1);
+    const uint32_t a_left = (a << 1) | (al >> 31), a_right = (a >> 1) | (ar << 31);
+#pragma unroll
+    for (int dy = -1; dy <= 1; dy += 2) {
+      const uint32_t ay = dy < 0 ? au : R.at(z, yz + 1, 0), by = dy < 0 ? bu : R.at(z + 1, yz + 1, 0);
+      const uint32_t qy = by & ~ay;
+      const uint32_t over = p & qy;
+      unite(over & ~(over << 1), dy * g.W);
+      const uint32_t free = p & ~by;
+      if (!free) continue;
+      const uint32_t qyl = R.at(z + 1, yz + dy, -1) & ~R.at(z, yz + dy, -1);
+      const uint32_t qyr = R.at(z + 1, yz + dy, 1) & ~R.at(z, yz + dy, 1);
+      unite(free & ~a_left & ((qy << 1) | (qyl >> 31)), dy * g.W - 1);
+      unite(free & ~a_right & ((qy >> 1) | (qyr << 31)), dy * g.W + 1);
+    }
   }
 }
 
@@ -121,32 +195,39 @@ __global__ void k_relabel(const uint32_t* m, MaskGeom g, int32_t* L, int32_t* st
   }
 }
 
-// F[label] = 1 for every seed voxel (benign races: every writer writes 1).
-// Seeds lie in phi2, so the voxels of a run of seeds in a row share one
-// component: only the first voxel of every run is looked up.
-__global__ void k_seed_flags(const uint32_t* seed, MaskGeom g, const int32_t* L, uint8_t* F) {
+// F[root] = 1 for the component of every seed, i.e. voxel of phi2 in N phi1
+// (benign races: every writer writes 1).  Seeds lie in phi2, so the voxels of
+// a run of seeds share one component: only the first voxel of every run is
+// looked up.  The union-find is walked from the voxel's key: labels of all
+// voxels would be a pass over the volume for these few.
+__global__ void k_seed_flags(const uint32_t* phi1, const uint32_t* phi2, MaskGeom g, int conn,
+                             int32_t* L, uint8_t* F, int32_t* status) {
   const long long nwords = (long long)g.H * g.Wp;
+  const int npx = g.H * g.W;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < nwords;
        i += (long long)gridDim.x * blockDim.x) {
     int y, w;
     split_index(i, g.Wp, y, w);
-    const uint32_t cur = __ldg(seed + i) & vmask(w, g.W);
-    const uint32_t prev = w > 0 ? __ldg(seed + i - 1) : 0u;
-    uint32_t bits = cur & ~((cur << 1) | (prev >> 31));
+    const uint32_t m = __ldg(phi2 + i) & vmask(w, g.W);
+    if (!m) continue;
+    const uint32_t seeds = near3_word(phi1, g, conn, y, w) & m;
+    uint32_t bits = seeds & ~(m & (seeds << 1));
     while (bits) {
       const int b = __ffs(bits) - 1;
       bits &= bits - 1;
-      const int lab = __ldg(L + (size_t)y * g.W + 32 * w + b);
-      if ((unsigned)lab < (unsigned)(g.H * g.W)) F[lab] = 1;
+      const int v = y * g.W + 32 * w + b;
+      const int root = g_find(L, ldcg(&L[v]), npx, status);
+      if (!__ldcg(F + root)) F[root] = 1;
     }
   }
 }
 
 // Z = the voxels of phi2 whose component is flagged: one lookup per run of
 // phi2 inside the word (a run is one component), the run's bits taken whole.
-__global__ void k_select_flagged(const uint32_t* phi2, MaskGeom g, const int32_t* L,
-                                 const uint8_t* F, uint32_t* Z) {
+__global__ void k_select_flagged(const uint32_t* phi2, MaskGeom g, int32_t* L, const uint8_t* F,
+                                 uint32_t* Z, int32_t* status) {
   const long long nwords = (long long)g.H * g.Wp;
+  const int npx = g.H * g.W;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < nwords;
        i += (long long)gridDim.x * blockDim.x) {
     int y, w;
@@ -159,8 +240,8 @@ __global__ void k_select_flagged(const uint32_t* phi2, MaskGeom g, const int32_t
       // the run: bits b.. up to the first clear bit
       const uint32_t from = bits >> b;
       const uint32_t len_mask = ~from ? ((~from & (0u - ~from)) - 1u) : 0xFFFFFFFFu;
-      const int lab = __ldg(L + (size_t)y * g.W + 32 * w + b);
-      if ((unsigned)lab < (unsigned)(g.H * g.W) && F[lab]) sel |= len_mask << b;
+      const int root = g_find(L, ldcg(&L[y * g.W + 32 * w + b]), npx, status);
+      if (__ldg(F + root)) sel |= len_mask << b;
     }
     Z[i] = sel;
   }
@@ -169,37 +250,42 @@ __global__ void k_select_flagged(const uint32_t* phi2, MaskGeom g, const int32_t
 }  // namespace
 
 cudaError_t launch_near3(const uint32_t* a, MaskGeom g, int conn, uint32_t* out, cudaStream_t st) {
-  k_near3<<<grid_for((long long)g.H * g.Wp, kThreads * 2), kThreads, 0, st>>>(a, g, conn, nullptr,
-                                                                            out);
+  k_near3<<<grid_for((long long)g.H * g.Wp, kThreads), kThreads, 0, st>>>(a, g, conn, out);
+  return cudaGetLastError();
+}
+
+// The union-find of a volume's components: every voxel's key leads to its
+// component's root, the minimum index of all its voxels.
+static cudaError_t launch_components3(const uint32_t* mask, MaskGeom g, int conn, CclScratch sc,
+                                      int32_t* status, cudaStream_t st) {
+  cudaError_t e = launch_ccl_labels(mask, g, conn == 26 ? 8 : 4, sc, status, st);
+  if (e) return e;
+  const int Hs = slice_rows(g), D = g.H / Hs;
+  if (D < 2) return cudaSuccess;
+  const long long words = (long long)(D - 1) * Hs * g.Wp;
+  k_zmerge<<<grid_for(words, kThreads), kThreads, 0, st>>>(mask, g, conn, sc.G, status);
   return cudaGetLastError();
 }
 
 cudaError_t launch_labels3(const uint32_t* mask, MaskGeom g, int conn, CclScratch sc,
                            int32_t* status, cudaStream_t st) {
-  cudaError_t e = launch_ccl_labels(mask, g, conn == 26 ? 8 : 4, sc, status, st);
-  if (e) return e;
-  const int Hs = slice_rows(g), D = g.H / Hs;
-  if (D < 2) return cudaSuccess;
-  const long long rows = (long long)(D - 1) * Hs;  // one warp per row pair
-  k_zmerge<<<grid_for(rows * 32, kThreads), kThreads, 0, st>>>(mask, g, conn, sc.G, status);
-  if ((e = cudaGetLastError())) return e;
+  cudaError_t e = launch_components3(mask, g, conn, sc, status, st);
+  if (e || g.H == slice_rows(g)) return e;
   k_relabel<<<grid_for((long long)g.H * g.W, kThreads * 4), kThreads, 0, st>>>(mask, g, sc.G, status);
   return cudaGetLastError();
 }
 
 cudaError_t launch_rz3(const uint32_t* phi1, const uint32_t* phi2, MaskGeom g, int conn,
                        Rz3Scratch sc, uint32_t* Z, int32_t* status, cudaStream_t st) {
-  cudaError_t e = launch_labels3(phi2, g, conn, sc.ccl, status, st);
+  cudaError_t e = launch_components3(phi2, g, conn, sc.ccl, status, st);
   if (e) return e;
-  // seeds: the voxels of phi2 in N phi1
-  k_near3<<<grid_for((long long)g.H * g.Wp, kThreads * 2), kThreads, 0, st>>>(phi1, g, conn, phi2,
-                                                                            sc.seed);
-  if ((e = cudaGetLastError())) return e;
   if ((e = cudaMemsetAsync(sc.F, 0, (size_t)g.H * g.W, st))) return e;
   const long long nwords = (long long)g.H * g.Wp;
-  k_seed_flags<<<grid_for(nwords, kThreads * 2), kThreads, 0, st>>>(sc.seed, g, sc.ccl.G, sc.F);
+  k_seed_flags<<<grid_for(nwords, kThreads), kThreads, 0, st>>>(phi1, phi2, g, conn, sc.ccl.G, sc.F,
+                                                                status);
   if ((e = cudaGetLastError())) return e;
-  k_select_flagged<<<grid_for(nwords, kThreads * 2), kThreads, 0, st>>>(phi2, g, sc.ccl.G, sc.F, Z);
+  k_select_flagged<<<grid_for(nwords, kThreads), kThreads, 0, st>>>(phi2, g, sc.ccl.G, sc.F, Z,
+                                                                    status);
   return cudaGetLastError();
 }
 
