@@ -905,28 +905,43 @@ vl_status plain_enqueue(vl_context* ctx, const Plan& P, vl_image* const* imgs, i
   for (int q = 0; q < P.n_roots; ++q) root_slot[P.exec_roots[q]] = P.root_slot[q];
   std::vector<uint32_t*> val(N, nullptr);
   std::vector<DevBlockPtr> own(N);
+  auto mask_for = [&](int i) {
+    if (root_slot[i] >= 0) {
+      val[i] = root_buf(root_slot[i]);
+      return cudaSuccess;
+    }
+    const cudaError_t z = dev_alloc(ctx, mask_bytes, st, &own[i]);
+    if (!z) val[i] = static_cast<uint32_t*>(own[i]->ptr);
+    return z;
+  };
+  std::map<std::pair<int, int>, std::vector<int>> thr;  // thresholds of a channel, last first
+  for (int i = N - 1; i >= 0; --i)
+    if (P.exec[i].op == E_THR || P.exec[i].op == E_PCT) thr[{P.exec[i].img, P.exec[i].ch}].push_back(i);
   for (int i = 0; i < N; ++i) {
     const ENode& x = P.exec[i];
     if (x.op == E_MASK) { val[i] = imgs[x.img]->mask; continue; }
-    if (root_slot[i] >= 0) {
-      val[i] = root_buf(root_slot[i]);
-    } else {
-      if ((e = dev_alloc(ctx, mask_bytes, st, &own[i]))) return cuda_err(ctx, e, "allocating a mask");
-      val[i] = static_cast<uint32_t*>(own[i]->ptr);
-    }
+    if (val[i]) continue;  // a threshold made along with an earlier one
+    if ((e = mask_for(i))) return cuda_err(ctx, e, "allocating a mask");
     uint32_t* o = val[i];
     switch (x.op) {
       case E_TRUE: e = launch_const(g, true, o, st); break;
       case E_FALSE: e = launch_const(g, false, o, st); break;
-      case E_THR: {
-        const Chan c = chan(x.img, x.ch);
-        e = launch_threshold(c.p, c.format, pitch, g, x.t, nullptr, x.lt, o, st);
-        break;
-      }
+      case E_THR:
       case E_PCT: {
+        // and the next ones of the same channel, in one pass over it
         const Chan c = chan(x.img, x.ch);
-        e = launch_threshold(c.p, c.format, pitch, g, 0.f, static_cast<float*>(pct->ptr) + x.pct_slot,
-                             x.lt, o, st);
+        ThrSet T{};
+        int n = 0;
+        for (std::vector<int>& todo = thr[{x.img, x.ch}]; n < THR_SET && !todo.empty(); ++n) {
+          const int k = todo.back();
+          todo.pop_back();
+          if (!val[k] && (e = mask_for(k))) return cuda_err(ctx, e, "allocating a mask");
+          const ENode& t = P.exec[k];
+          T.job[n] = ThrSet::Job{t.t, t.lt ? 1 : 0,
+                                 t.op == E_PCT ? static_cast<float*>(pct->ptr) + t.pct_slot : nullptr,
+                                 val[k]};
+        }
+        e = launch_thresholds(c.p, c.format, g, T, n, st);
         break;
       }
       case E_NOT: e = launch_not(val[x.a], g, o, st); break;

@@ -73,6 +73,37 @@ VL_DEV uint32_t near_word(uint32_t ul, uint32_t uc, uint32_t ur, uint32_t ml,
   return uc | dc | hdil(ml, mc, mr);
 }
 
+// N on a vector of four words x, given the words left and right of it in the
+// row: for the square, of the three rows around together (o = x); for the
+// cross, of its own row, with o the rows above and below.
+VL_DEV uint4 near_vec(uint4 x, uint4 o, uint32_t l, uint32_t e) {
+  return make_uint4(o.x | hdil(l, x.x, x.y), o.y | hdil(x.x, x.y, x.z), o.z | hdil(x.y, x.z, x.w),
+                    o.w | hdil(x.z, x.w, e));
+}
+VL_DEV uint4 or4(uint4 a, uint4 b) { return make_uint4(a.x | b.x, a.y | b.y, a.z | b.z, a.w | b.w); }
+// Vector jv of a row without the bits that are no pixels.
+VL_DEV uint4 clip_vec(uint4 v, int jv, int W) {
+  if (128 * (jv + 1) <= W) return v;
+  return make_uint4(v.x & vmask(4 * jv, W), v.y & vmask(4 * jv + 1, W), v.z & vmask(4 * jv + 2, W),
+                    v.w & vmask(4 * jv + 3, W));
+}
+
+// The 8 lanes of a group hold the nibbles n[u] of four 32-pixel words u (lane
+// `sub` pixels 4 * sub ..): returns word sub >> 1.  Three shuffles: half of
+// the words change sides with the other four lanes, then one of two with the
+// lane two further, then the halves of a word are joined.
+VL_DEV uint32_t join_nibbles4(const uint32_t (&n)[4], int sub) {
+  const int h = 4 * (sub & 3);
+  const uint32_t x = (n[0] | n[1] << 16) << h, y = (n[2] | n[3] << 16) << h;
+  const bool high = sub & 4, second = sub & 2;
+  const uint32_t own = high ? y : x, other = __shfl_xor_sync(0xFFFFFFFFu, high ? x : y, 4);
+  const uint32_t lo = high ? other : own, hi = high ? own : other;
+  const uint32_t w0 = __byte_perm(lo, hi, 0x5410), w1 = __byte_perm(lo, hi, 0x7632);
+  uint32_t w = second ? w1 : w0;
+  w |= __shfl_xor_sync(0xFFFFFFFFu, second ? w0 : w1, 2);
+  return w | __shfl_xor_sync(0xFFFFFFFFu, w, 1);
+}
+
 // Order-preserving map float -> uint32 (for selects on float keys); every
 // NaN maps to the largest key, after +infinity.
 VL_DEV uint32_t f2key(float f) {

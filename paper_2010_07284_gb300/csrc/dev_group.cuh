@@ -254,13 +254,6 @@ VL_DEV uint4 rank_result(uint4 w, uint4 nan, bool lt) {
   return make_uint4((w.x ^ f) & ~nan.x, (w.y ^ f) & ~nan.y, (w.z ^ f) & ~nan.z, (w.w ^ f) & ~nan.w);
 }
 
-// N on vector q, given the words left and right of it in the row (conn 4),
-// or of the three rows around together (conn 8).
-VL_DEV uint4 near_vec(uint4 x, uint4 o, uint32_t l, uint32_t e) {
-  return make_uint4(o.x | hdil(l, x.x, x.y), o.y | hdil(x.x, x.y, x.z), o.z | hdil(x.y, x.z, x.w),
-                    o.w | hdil(x.z, x.w, e));
-}
-
 // The value of instruction I (no load, store or float threshold) on vector q.
 // stage: the thread's place in the staged planes.
 template <bool ALIGNED>

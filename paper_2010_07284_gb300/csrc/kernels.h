@@ -18,9 +18,20 @@ inline __host__ __device__ int slice_rows(const MaskGeom& g) { return g.Hs > 0 ?
 inline __host__ __device__ int ccl_rows(const MaskGeom& g) { return g.cth > 0 ? g.cth : CCL_TH; }
 
 // ---- plain per-operator kernels (one launch per primitive) ----
-// `plane`: one channel of H x pitch elements, float or uint16 by `format`.
-cudaError_t launch_threshold(const void* plane, int format, int pitch, MaskGeom g, float t,
-                             const float* t_dev, bool lt, uint32_t* out, cudaStream_t st);
+// (Masks: 16-byte aligned.)
+// n (1 .. THR_SET) thresholds of one channel, H rows of 32 * Wp elements, float
+// or uint16 by `format`; t_dev, unless null, holds the bound in place of t.
+constexpr int THR_SET = 4;
+struct ThrSet {
+  struct Job {
+    float t;
+    int lt;
+    const float* t_dev;
+    uint32_t* out;
+  } job[THR_SET];
+};
+cudaError_t launch_thresholds(const void* plane, int format, MaskGeom g, const ThrSet& T, int n,
+                              cudaStream_t st);
 cudaError_t launch_not(const uint32_t* a, MaskGeom g, uint32_t* out, cudaStream_t st);
 cudaError_t launch_and(const uint32_t* a, const uint32_t* b, MaskGeom g, uint32_t* out,
                        cudaStream_t st);
