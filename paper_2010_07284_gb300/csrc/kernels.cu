@@ -242,6 +242,24 @@ __global__ void k_unpack_u8(const uint32_t* __restrict__ src, MaskGeom g, uint8_
   }
 }
 
+// n vectors from src to dst.  Launched so that it may come up while the kernel
+// before it ends: it waits for that one's results, and then lets the next one
+// come up.
+constexpr int COPY_UNR = 4;
+__global__ void __launch_bounds__(kThreads) k_copy(const uint4* __restrict__ src, uint4* __restrict__ dst,
+                                                   unsigned n) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const unsigned first = blockIdx.x * (kThreads * COPY_UNR) + threadIdx.x;
+  uint4 v[COPY_UNR];
+#pragma unroll
+  for (int u = 0; u < COPY_UNR; ++u)
+    if (first + u * kThreads < n) v[u] = __ldcg(src + first + u * kThreads);
+#pragma unroll
+  for (int u = 0; u < COPY_UNR; ++u)
+    if (first + u * kThreads < n) dst[first + u * kThreads] = v[u];
+}
+
 __global__ void k_clear_padding(uint32_t* m, MaskGeom g) {
   const long long nwords = (long long)g.H * g.Wp;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < nwords;
@@ -432,6 +450,22 @@ cudaError_t launch_pack_u8(const uint8_t* src, MaskGeom g, uint32_t* out, cudaSt
 cudaError_t launch_unpack_u8(const uint32_t* src, MaskGeom g, uint8_t* out, cudaStream_t st) {
   k_unpack_u8<<<grid_for((long long)g.H * g.W, kThreads * 8), kThreads, 0, st>>>(src, g, out);
   return cudaGetLastError();
+}
+cudaError_t launch_copy(const void* src, void* dst, size_t bytes, cudaStream_t st) {
+  const size_t n = bytes / 16, per_block = (size_t)kThreads * COPY_UNR;
+  if (bytes % 16 || n > 0x7FFFFFFFu) return cudaErrorInvalidValue;
+  if (!n) return cudaSuccess;
+  cudaLaunchAttribute early{};
+  early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  early.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)((n + per_block - 1) / per_block));
+  cfg.blockDim = dim3(kThreads);
+  cfg.stream = st;
+  cfg.attrs = &early;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k_copy, static_cast<const uint4*>(src), static_cast<uint4*>(dst),
+                            (unsigned)n);
 }
 cudaError_t launch_clear_padding(uint32_t* m, MaskGeom g, cudaStream_t st) {
   k_clear_padding<<<grid_for((long long)g.H * g.Wp, kThreads * 4), kThreads, 0, st>>>(m, g);

@@ -111,6 +111,8 @@ cudaError_t launch_rz3(const uint32_t* phi1, const uint32_t* phi2, MaskGeom g, i
 // ---- mask conversion ----
 cudaError_t launch_pack_u8(const uint8_t* src, MaskGeom g, uint32_t* out, cudaStream_t st);
 cudaError_t launch_unpack_u8(const uint32_t* src, MaskGeom g, uint8_t* out, cudaStream_t st);
+// A copy within the device, both ends 16-byte aligned, bytes a multiple of 16.
+cudaError_t launch_copy(const void* src, void* dst, size_t bytes, cudaStream_t st);
 cudaError_t launch_clear_padding(uint32_t* m, MaskGeom g, cudaStream_t st);
 
 // ---- the paper's pointer-jumping labelling (comparison only) ----
