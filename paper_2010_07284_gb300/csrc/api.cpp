@@ -183,8 +183,8 @@ bool copy_kernel_takes(const vl_context* ctx, const void* dst, size_t bytes) {
 }
 // Masks up to this size are copied by a kernel: back to back on a stream it
 // takes 0.8 us for the 7.7 KB of a 240 x 240 mask, 1.2 us for 512 KB and 2.2 us
-// for 4 MB (each comes up while the one before ends), the runtime's copy 2.9,
-// 4.1 and 8.2 us.
+// for 4 MB (each comes up while the one before ends), the runtime's copy 4.1 us
+// for each of them; from 8 MB on the two are alike.
 constexpr size_t kCopyKernelBytes = 4 << 20;
 
 int ccl_merge_chunks(int H, int Wp, int cth) {

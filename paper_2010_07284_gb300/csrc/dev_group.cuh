@@ -139,27 +139,22 @@ constexpr uint32_t P_PUT = 1u << 23;   // the next instruction stores this value
 constexpr uint32_t P_SYNC = 0x80u;     // with the opcode: a block barrier precedes
 constexpr uint32_t TH_LT = 1u << 29, TH_U16 = 1u << 30, TH_WRITTEN = 1u << 31;
 
-// The 32-pixel word whose nibbles the 8 lanes of its group hold.
-VL_DEV uint32_t join_nibbles(uint32_t nib, int sub) {
-  uint32_t word = nib << (4 * sub);
-  word |= __shfl_xor_sync(0xFFFFFFFFu, word, 1);
-  word |= __shfl_xor_sync(0xFFFFFFFFu, word, 2);
-  word |= __shfl_xor_sync(0xFFFFFFFFu, word, 4);
-  return word;
-}
-
 // A float threshold (a constant, or a percentile found earlier in the launch)
-// into buffer d: the rows it is needed on, the core words, and the one left
-// and right of them if a neighbour will be read (h > 0).  A lane loads 4
-// pixels (16 bytes, or 8 of uint16), a warp 4 words a load and UNR loads in
-// flight; the 8 lanes of a word merge their nibbles with three shuffles.
-// By the whole block.  Not inlined: the interpreter's loop needs its
-// registers.
+// into buffer d: the rows it is needed on, the tile's words that lie in the
+// image, and the one left and right of them if a neighbour will be read (h >
+// 0); further words lie outside the image, and nothing inside comes of them.
+// A lane loads 4 pixels (16 bytes, or 8 of uint16), a warp 4 words a load and
+// UNR loads in flight; three shuffles put four of them together.  By the whole
+// block.  Not inlined: the interpreter's loop needs its registers.
+//
+// Bound by the latency of its loads: the groups of 1024 slices (six thresholds a
+// pixel) take 877 us of the grid, and took 1157 with four loads in flight,
+// twelve shuffles, a division a load, and words outside the image.
 static __device__ __noinline__ void group_threshold(const DevJob& J, const StepDesc& S, int sub,
                                                     uint4 I, uint32_t* d) {
-  constexpr int UNR = 4;
+  constexpr int UNR = 8;
   const GroupGeom g = group_geom(J, S, sub);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, part = lane & 7;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, part = lane & 7, quad = lane >> 3;
   const int H = J.H, W = J.W, Wp = J.Wp, pitch = J.pitch, h = (I.y >> 16) & 0x7F;
   const void* plane = reinterpret_cast<const void*>(
       (unsigned long long)I.z | (unsigned long long)(I.w & 0xFFFFFFu) << 32);
@@ -167,26 +162,33 @@ static __device__ __noinline__ void group_threshold(const DevJob& J, const StepD
   const bool nc = !(I.w & TH_WRITTEN), lt = I.w & TH_LT;
   const float t = __uint_as_float((I.x >> 16) << 16 | (I.y & 0xFFFFu));
   const int side = h > 0 ? 1 : 0;
-  const int bw = J.gtww + 2 * side;  // words worked on in a row
+  const int bw = g.tww + 2 * side;  // words worked on in a row
   const int n = (g.th + 2 * h) * bw, y0 = g.r0 - h, w0 = g.w0 - side;
+  // idx / bw as a product (exact: idx * bw < 2^32)
+  const unsigned inv = bw > 1 ? 0xFFFFFFFFu / (unsigned)bw + 1u : 0u;
+  auto row_of = [&](int idx) { return bw > 1 ? (int)__umulhi((unsigned)idx, inv) : idx; };
   d += (g.halo - h) * g.nv * 4 + 4 - side;
   for (int base = warp * 4 * UNR; base < n; base += EXEC_WARPS * 4 * UNR) {
     float4 v[UNR];
 #pragma unroll
     for (int u = 0; u < UNR; ++u) {
-      const int idx = base + 4 * u + (lane >> 3), i = idx / bw, wg = w0 + idx - i * bw, y = y0 + i;
+      const int idx = base + 4 * u + quad, i = row_of(idx), wg = w0 + idx - i * bw, y = y0 + i;
       v[u] = idx < n && y >= 0 && y < H && wg >= 0 && wg < Wp
                  ? ld_px4(plane, fmt, nc, (size_t)y * pitch + 32 * wg + 4 * part)
                  : make_float4(t, t, t, t);  // (passes neither test)
     }
 #pragma unroll
-    for (int u = 0; u < UNR; ++u) {
-      const float4 x = v[u];
-      const uint32_t nib = lt ? ((x.x < t) | ((x.y < t) << 1) | ((x.z < t) << 2) | ((x.w < t) << 3))
-                              : ((x.x > t) | ((x.y > t) << 1) | ((x.z > t) << 2) | ((x.w > t) << 3));
-      const uint32_t word = join_nibbles(nib, part);
-      const int idx = base + 4 * u + (lane >> 3), i = idx / bw, j = idx - i * bw;
-      if (part == 0 && idx < n)
+    for (int u0 = 0; u0 < UNR; u0 += 4) {
+      uint32_t nib[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const float4 x = v[u0 + u];
+        nib[u] = lt ? ((x.x < t) | ((x.y < t) << 1) | ((x.z < t) << 2) | ((x.w < t) << 3))
+                    : ((x.x > t) | ((x.y > t) << 1) | ((x.z > t) << 2) | ((x.w > t) << 3));
+      }
+      const uint32_t word = join_nibbles4(nib, part);
+      const int idx = base + 4 * (u0 + (part >> 1)) + quad, i = row_of(idx), j = idx - i * bw;
+      if (!(part & 1) && idx < n)
         d[i * g.nv * 4 + j] = w0 + j >= 0 ? word & vmask(w0 + j, W) : 0u;
     }
   }
