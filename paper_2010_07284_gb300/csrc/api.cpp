@@ -327,19 +327,16 @@ vl_status batch_build(vl_context* ctx, const vl_job* jobs, int n_jobs, cudaStrea
   const bool split_selects = n_selects > 0 && n_selects < grid && select_px >= (1 << 18);
   std::vector<DevSteps> F;
   for (const Plan* P : formulas) F.push_back(device_steps(*P, split_selects));
-  std::vector<size_t> f_steps(formulas.size()), f_insns(formulas.size()), f_rz(formulas.size()),
+  std::vector<size_t> f_insns(formulas.size()), f_rz(formulas.size()),
       f_pct(formulas.size()), f_rtab(formulas.size()), f_rvals(formulas.size()),
-      f_doff(formulas.size()), f_deps(formulas.size()), f_arith(formulas.size());
+      f_arith(formulas.size());
   for (size_t k = 0; k < formulas.size(); ++k) {
     const Plan* P = formulas[k];
-    f_steps[k] = take(sizeof(StepDesc) * std::max<size_t>(1, F[k].steps.size()));
     f_insns[k] = take(sizeof(Insn) * std::max<size_t>(1, P->insns.size()));
     f_rz[k] = take(sizeof(RzDesc) * std::max<size_t>(1, P->rz.size()));
     f_pct[k] = take(sizeof(PctDesc) * std::max<size_t>(1, P->pct.size()));
     f_rtab[k] = take(sizeof(RankTab) * std::max<size_t>(1, P->rtab.size()));
     f_rvals[k] = take(sizeof(float) * std::max<size_t>(1, P->rvals.size()));
-    f_doff[k] = take(sizeof(int32_t) * std::max<size_t>(1, F[k].dep_off.size()));
-    f_deps[k] = take(sizeof(int32_t) * std::max<size_t>(1, F[k].deps.size()));
     f_arith[k] = take(sizeof(ArithInsn) * std::max<size_t>(1, P->arith.size()));
   }
   int total_steps = 0;
@@ -455,7 +452,14 @@ vl_status batch_build(vl_context* ctx, const vl_job* jobs, int n_jobs, cudaStrea
       return set_err(ctx, VL_ERR_INTERNAL, "internal: step order");
   }
   const size_t off_items = take(sizeof(WorkItem) * std::max<size_t>(1, items.size()));
-  const size_t off_need = take(sizeof(int32_t) * std::max(1, total_steps));
+  const size_t off_recs = take(sizeof(StepRec) * std::max(1, total_steps));
+  size_t n_more = 0;  // dependencies that do not fit the steps' records
+  for (int j = 0; j < n_jobs; ++j) {
+    const DevSteps& D = F[J[j].formula_idx];
+    for (size_t q = 0; q < D.steps.size(); ++q)
+      n_more += std::max(0, D.dep_off[q + 1] - D.dep_off[q] - REC_DEPS);
+  }
+  const size_t off_more = take(sizeof(StepRec::Dep) * std::max<size_t>(1, n_more));
   // counters: head, done[steps] -- zeroed before every run
   // (and the state of selects that many blocks share)
   const size_t off_counters = take(sizeof(int32_t) * (1 + total_steps));
@@ -511,27 +515,24 @@ vl_status batch_build(vl_context* ctx, const vl_job* jobs, int n_jobs, cudaStrea
   std::vector<char> host(tables_end, 0);
   for (size_t k = 0; k < formulas.size(); ++k) {
     const Plan* P = formulas[k];
-    const DevSteps& D = F[k];
-    if (!D.steps.empty()) std::memcpy(&host[f_steps[k]], D.steps.data(), sizeof(StepDesc) * D.steps.size());
     // on the device a group's pct_cnt counts its float thresholds, pct_off its loads
-    StepDesc* hs = reinterpret_cast<StepDesc*>(&host[f_steps[k]]);
-    for (size_t q = 0; q < D.steps.size(); ++q)
-      for (int i = 0; hs[q].kind == SK_GROUP && i < hs[q].insn_cnt; ++i) {
-        const int op = insn_op(P->insns[hs[q].insn_off + i]);
-        hs[q].pct_cnt += op == I_THR;
-        hs[q].pct_off += op == I_LOAD;
+    for (StepDesc& q : F[k].steps)
+      for (int i = 0; q.kind == SK_GROUP && i < q.insn_cnt; ++i) {
+        const int op = insn_op(P->insns[q.insn_off + i]);
+        q.pct_cnt += op == I_THR;
+        q.pct_off += op == I_LOAD;
       }
     if (!P->insns.empty()) std::memcpy(&host[f_insns[k]], P->insns.data(), sizeof(Insn) * P->insns.size());
     if (!P->rz.empty()) std::memcpy(&host[f_rz[k]], P->rz.data(), sizeof(RzDesc) * P->rz.size());
     if (!P->pct.empty()) std::memcpy(&host[f_pct[k]], P->pct.data(), sizeof(PctDesc) * P->pct.size());
     if (!P->rtab.empty()) std::memcpy(&host[f_rtab[k]], P->rtab.data(), sizeof(RankTab) * P->rtab.size());
     if (!P->rvals.empty()) std::memcpy(&host[f_rvals[k]], P->rvals.data(), sizeof(float) * P->rvals.size());
-    if (!D.dep_off.empty()) std::memcpy(&host[f_doff[k]], D.dep_off.data(), sizeof(int32_t) * D.dep_off.size());
-    if (!D.deps.empty()) std::memcpy(&host[f_deps[k]], D.deps.data(), sizeof(int32_t) * D.deps.size());
     if (!P->arith.empty()) std::memcpy(&host[f_arith[k]], P->arith.data(), sizeof(ArithInsn) * P->arith.size());
   }
   DevJob* hj = reinterpret_cast<DevJob*>(&host[off_jobs]);
-  int32_t* hneed = reinterpret_cast<int32_t*>(&host[off_need]);
+  StepRec* hrec = reinterpret_cast<StepRec*>(&host[off_recs]);
+  StepRec::Dep* hmore = reinterpret_cast<StepRec::Dep*>(&host[off_more]);
+  int32_t more = 0;
   int32_t* counters_dev = reinterpret_cast<int32_t*>(tb + off_counters);
   int32_t* status_dev = reinterpret_cast<int32_t*>(pb + off_status);
   for (int j = 0; j < n_jobs; ++j) {
@@ -574,9 +575,6 @@ vl_status batch_build(vl_context* ctx, const vl_job* jobs, int n_jobs, cudaStrea
     d.n_root_slots = P.n_root_slots;
     const int k = I.formula_idx;
     d.insns = reinterpret_cast<const Insn*>(tb + f_insns[k]);
-    d.steps = reinterpret_cast<const StepDesc*>(tb + f_steps[k]);
-    d.dep_off = reinterpret_cast<const int32_t*>(tb + f_doff[k]);
-    d.deps = reinterpret_cast<const int32_t*>(tb + f_deps[k]);
     d.rz = reinterpret_cast<const RzDesc*>(tb + f_rz[k]);
     d.pct = reinterpret_cast<const PctDesc*>(tb + f_pct[k]);
     d.pct_val = reinterpret_cast<float*>(tb + I.off_pct);
@@ -593,9 +591,24 @@ vl_status batch_build(vl_context* ctx, const vl_job* jobs, int n_jobs, cudaStrea
     d.c_th = I.cth;
     d.status = status_dev + j;
     hj[j] = d;
-    for (size_t s = 0; s < I.need.size(); ++s) hneed[I.step_base + s] = I.need[s];
+    const DevSteps& D = F[I.formula_idx];
+    for (size_t q = 0; q < D.steps.size(); ++q) {
+      StepRec r{};
+      r.step = D.steps[q];
+      if (r.step.kind == SK_RZ_LOCAL || r.step.kind == SK_RZ_MERGE || r.step.kind == SK_RZ_FINAL)
+        r.per_rz = I.need[q] / r.step.rz_cnt;
+      r.n_deps = D.dep_off[q + 1] - D.dep_off[q];
+      r.more = more;
+      for (int i = 0; i < r.n_deps; ++i) {
+        const int dep = D.deps[D.dep_off[q] + i];
+        const StepRec::Dep e{I.step_base + dep, I.need[dep]};
+        if (i < REC_DEPS) r.dep[i] = e;
+        else hmore[more++] = e;
+      }
+      hrec[I.step_base + q] = r;
+    }
   }
-  // items with job-relative steps
+  for (WorkItem& it : items) it.step += J[it.job].step_base;
   if (!items.empty()) std::memcpy(&host[off_items], items.data(), sizeof(WorkItem) * items.size());
   e = cudaMemcpyAsync(tb, host.data(), tables_end, cudaMemcpyHostToDevice, st);
   if (e) return cuda_err(ctx, e, "uploading batch tables");
@@ -610,7 +623,8 @@ vl_status batch_build(vl_context* ctx, const vl_job* jobs, int n_jobs, cudaStrea
   L.n_items = (int32_t)items.size();
   L.head = counters_dev;
   L.done = counters_dev + 1;
-  L.need = reinterpret_cast<const int32_t*>(tb + off_need);
+  L.steps = reinterpret_cast<const StepRec*>(tb + off_recs);
+  L.more_deps = reinterpret_cast<const StepRec::Dep*>(tb + off_more);
   L.spin_limit = ctx->cfg.spin_limit != 0 ? ctx->cfg.spin_limit : (1LL << 22);
   L.group_buffers = ctx->nb;
   L.grid = std::max(1, std::min<int>(grid, (int)items.size()));

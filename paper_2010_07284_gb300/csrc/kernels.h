@@ -131,7 +131,8 @@ struct ExecLaunch {
   int32_t n_items;
   int32_t* head;           // work-queue head (zeroed before launch)
   int32_t* done;           // per (job, step) finished sub-items (zeroed)
-  const int32_t* need;     // per (job, step) sub-items in total
+  const StepRec* steps;    // per (job, step)
+  const StepRec::Dep* more_deps;
   int64_t spin_limit;
   int32_t group_buffers;   // shared-memory buffers per group tile
   int32_t grid;            // CTAs

@@ -57,7 +57,7 @@ int64_t estimate_bytes(const Plan& P, int H, int W) {
   b += (size_t)P.n_scratch_sets *
        (align256(2 * px * 4) + align256(tstate * 4) + align256(tstate));
   b += align256(sizeof(uint32_t) * SEL_HIST * P.pct.size());
-  b += align256(sizeof(Insn) * P.insns.size()) + align256(sizeof(StepDesc) * P.steps.size()) +
+  b += align256(sizeof(Insn) * P.insns.size()) + align256(sizeof(StepRec) * (P.steps.size() + SEL_PASSES)) +
        64 * 1024;
   return (int64_t)b;
 }

@@ -232,9 +232,6 @@ struct DevJob {
   uint32_t* root_mem;
   int32_t n_inter_slots, n_root_slots;
   const Insn* insns;
-  const StepDesc* steps;        // this job's formula steps
-  const int32_t* dep_off;       // step dependencies (CSR, job-relative steps)
-  const int32_t* deps;
   const RzDesc* rz;
   const PctDesc* pct;
   float* pct_val;               // percentile values by slot
@@ -266,11 +263,25 @@ VL_HD_INLINE int32_t* rz_state(const DevJob& J, int k) {
   return reinterpret_cast<int32_t*>(J.rzs + k * J.set_bytes + J.off_state);
 }
 
+// A step of a job as the executor takes it up, in one load of a warp: what it
+// is, and which steps (of the launch) it waits for until they have done how
+// many sub-items.
+constexpr int REC_DEPS = 8;
+struct StepRec {
+  StepDesc step;
+  int32_t per_rz;      // rho batches: sub-items of each
+  int32_t n_deps;
+  int32_t more;        // dependencies beyond REC_DEPS: the first, in the launch's list
+  int32_t pad[2];
+  struct Dep { int32_t step, need; } dep[REC_DEPS];
+};
+static_assert(sizeof(StepRec) == 128, "a word per lane");
+
 // One work item of the persistent executor: a range of `count` consecutive
 // sub-items (tiles, chunks, rz x tile) of one step of one job.
 struct WorkItem {
   int32_t job;
-  int32_t step;        // step index within the job
+  int32_t step;        // step index within the job; on the device, of the launch
   int32_t first;       // first sub-item
   int32_t count;       // sub-items in this item
 };
