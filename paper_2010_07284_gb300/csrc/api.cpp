@@ -961,41 +961,76 @@ vl_status plain_enqueue(vl_context* ctx, const Plan& P, vl_image* const* imgs, i
     if (x.b >= 0 && (x.op == E_AND || x.op == E_OR || x.op == E_ANDNOT || x.op == E_RZ)) uses[x.b]++;
   }
   for (int q = 0; q < P.n_roots; ++q) root_slot[P.exec_roots[q]] = P.root_slot[q];
-  std::vector<uint32_t*> val(N, nullptr);
-  std::vector<DevBlockPtr> own(N);
-  auto mask_for = [&](int i) {
-    if (root_slot[i] >= 0) {
-      val[i] = root_buf(root_slot[i]);
-      return cudaSuccess;
+  // thresholds of a channel, in sets of up to THR_SET that one pass makes at
+  // the first one's place
+  std::vector<std::vector<int>> sets;
+  std::vector<int> set_of(N, -1);
+  {
+    std::map<std::pair<int, int>, int> open;  // channel -> its last set
+    for (int i = 0; i < N; ++i) {
+      const ENode& x = P.exec[i];
+      if (x.op != E_THR && x.op != E_PCT) continue;
+      const auto at = open.find({x.img, x.ch});
+      if (at == open.end() || (int)sets[at->second].size() == THR_SET) {
+        open[{x.img, x.ch}] = set_of[i] = (int)sets.size();
+        sets.push_back({i});
+      } else {
+        set_of[i] = at->second;
+        sets[at->second].push_back(i);
+      }
     }
-    const cudaError_t z = dev_alloc(ctx, mask_bytes, st, &own[i]);
-    if (!z) val[i] = static_cast<uint32_t*>(own[i]->ptr);
-    return z;
-  };
-  std::map<std::pair<int, int>, std::vector<int>> thr;  // thresholds of a channel, last first
-  for (int i = N - 1; i >= 0; --i)
-    if (P.exec[i].op == E_THR || P.exec[i].op == E_PCT) thr[{P.exec[i].img, P.exec[i].ch}].push_back(i);
+  }
+  // one block for the intermediate masks: a place per mask alive at a time
+  std::vector<int> place(N, -1);
+  int places = 0;
+  {
+    std::vector<int> left = uses, free_places;
+    auto take = [&](int i) {
+      if (root_slot[i] >= 0) return;
+      if (free_places.empty()) free_places.push_back(places++);
+      place[i] = free_places.back();
+      free_places.pop_back();
+    };
+    auto give = [&](int v) {
+      if (v >= 0 && --left[v] == 0 && place[v] >= 0) free_places.push_back(place[v]);
+    };
+    for (int i = 0; i < N; ++i) {
+      const ENode& x = P.exec[i];
+      if (x.op == E_MASK) continue;
+      if (set_of[i] < 0) take(i);
+      else if (sets[set_of[i]][0] == i) for (int k : sets[set_of[i]]) take(k);
+      const bool bin = x.op == E_AND || x.op == E_OR || x.op == E_ANDNOT || x.op == E_RZ;
+      if (bin || x.op == E_NOT || x.op == E_NEAR || x.op == E_COPY) give(x.a);
+      if (bin) give(x.b);
+    }
+  }
+  const size_t place_bytes = align_up(mask_bytes, 256);
+  DevBlockPtr masks;
+  if (places && (e = dev_alloc(ctx, place_bytes * places, st, &masks)))
+    return cuda_err(ctx, e, "allocating the masks");
+  std::vector<uint32_t*> val(N, nullptr);
   for (int i = 0; i < N; ++i) {
     const ENode& x = P.exec[i];
-    if (x.op == E_MASK) { val[i] = imgs[x.img]->mask; continue; }
-    if (val[i]) continue;  // a threshold made along with an earlier one
-    if ((e = mask_for(i))) return cuda_err(ctx, e, "allocating a mask");
+    if (x.op == E_MASK) val[i] = imgs[x.img]->mask;
+    else if (root_slot[i] >= 0) val[i] = root_buf(root_slot[i]);
+    else val[i] = reinterpret_cast<uint32_t*>(static_cast<char*>(masks->ptr) + place_bytes * place[i]);
+  }
+  for (int i = 0; i < N; ++i) {
+    const ENode& x = P.exec[i];
+    if (x.op == E_MASK || (set_of[i] >= 0 && sets[set_of[i]][0] != i)) continue;
     uint32_t* o = val[i];
     switch (x.op) {
       case E_TRUE: e = launch_const(g, true, o, st); break;
       case E_FALSE: e = launch_const(g, false, o, st); break;
       case E_THR:
       case E_PCT: {
-        // and the next ones of the same channel, in one pass over it
         const Chan c = chan(x.img, x.ch);
         ThrSet T{};
-        int n = 0;
-        for (std::vector<int>& todo = thr[{x.img, x.ch}]; n < THR_SET && !todo.empty(); ++n) {
-          const int k = todo.back();
-          todo.pop_back();
-          if (!val[k] && (e = mask_for(k))) return cuda_err(ctx, e, "allocating a mask");
+        const int n = (int)sets[set_of[i]].size();
+        for (int j = 0; j < n; ++j) {
+          const int k = sets[set_of[i]][j];
           const ENode& t = P.exec[k];
-          T.job[n] = ThrSet::Job{t.t, t.lt ? 1 : 0,
+          T.job[j] = ThrSet::Job{t.t, t.lt ? 1 : 0,
                                  t.op == E_PCT ? static_cast<float*>(pct->ptr) + t.pct_slot : nullptr,
                                  val[k]};
         }
@@ -1017,13 +1052,6 @@ vl_status plain_enqueue(vl_context* ctx, const Plan& P, vl_image* const* imgs, i
       default: return set_err(ctx, VL_ERR_INTERNAL, "plain form: unknown node");
     }
     if (e) return cuda_err(ctx, e, "launching a plain operator");
-    auto release = [&](int v) {
-      if (v >= 0 && --uses[v] == 0 && own[v]) { own[v].reset(); }
-    };
-    const bool bin = x.op == E_AND || x.op == E_OR || x.op == E_ANDNOT || x.op == E_RZ;
-    const bool un = x.op == E_NOT || x.op == E_NEAR || x.op == E_COPY;
-    if (un || bin) release(x.a);
-    if (bin) release(x.b);
   }
   return VL_OK;
 }

@@ -7,6 +7,7 @@
 #include "dev_common.cuh"
 #include "dev_select.cuh"
 #include "kernels.h"
+#include "launch.cuh"
 
 namespace vl {
 
@@ -31,11 +32,12 @@ int grid_for(long long items, int per_block, int cap = 152 * 32) {
 // (3.8 TB/s, launch included), where one pass each with two loads in flight
 // and twelve shuffles took 15 us a threshold.
 template <int N>
-__global__ void __launch_bounds__(kThreads) k_thresholds(const void* __restrict__ plane, int format,
+__global__ void __launch_bounds__(kThreads) k_thresholds(const void* plane, int format,
                                                          MaskGeom g, const __grid_constant__ ThrSet T) {
+  grid_wait(plane);
   float t[N];
 #pragma unroll
-  for (int k = 0; k < N; ++k) t[k] = T.job[k].t_dev ? __ldg(T.job[k].t_dev) : T.job[k].t;
+  for (int k = 0; k < N; ++k) t[k] = T.job[k].t_dev ? __ldcg(T.job[k].t_dev) : T.job[k].t;
   const int lane = threadIdx.x & 31, sub = lane & 7, group = lane >> 3;
   const long long nwords = (long long)g.H * g.Wp;
   const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
@@ -68,8 +70,9 @@ __global__ void __launch_bounds__(kThreads) k_thresholds(const void* __restrict_
 // Masks are rows of Wp / 4 vectors of four words; a thread takes one at a time
 // (a word at a time, NOT took 5.3 us on 155 x 240 x 240 and takes 3.4).
 template <int OP>  // 0 not, 1 and, 2 or, 3 const false, 4 const true, 5 and-not
-__global__ void k_pointwise(const uint4* __restrict__ a, const uint4* __restrict__ b, MaskGeom g,
-                            uint4* __restrict__ out) {
+__global__ void k_pointwise(const uint4* a, const uint4* b, MaskGeom g,
+                            uint4* out) {
+  grid_wait(a, b);
   const int nv = g.Wp >> 2;
   const long long n = (long long)g.H * nv;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
@@ -92,7 +95,8 @@ __global__ void k_pointwise(const uint4* __restrict__ a, const uint4* __restrict
   }
 }
 
-__global__ void k_near(const uint32_t* __restrict__ a, MaskGeom g, int conn, uint4* __restrict__ out) {
+__global__ void k_near(const uint32_t* a, MaskGeom g, int conn, uint4* out) {
+  grid_wait(a);
   const int nv = g.Wp >> 2;
   const long long n = (long long)g.H * nv;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
@@ -129,13 +133,15 @@ struct SelBatch {
 __global__ void __launch_bounds__(EXEC_THREADS, 2)
 k_sel_pass(const __grid_constant__ SelBatch B, int pass) {
   __shared__ __align__(16) SelectSmem s;
-  const SelJob j = B.job[blockIdx.y];
+  SelJob j = B.job[blockIdx.y];
+  grid_wait(j.plane);
   sel_pass(s, SelChan{j.plane, j.format, 1, B.H, B.W, B.pitch}, pass, blockIdx.x, gridDim.x, j.rank,
            B.state + (size_t)blockIdx.y * SEL_HIST);
 }
 __global__ void __launch_bounds__(EXEC_THREADS) k_sel_finish(const __grid_constant__ SelBatch B) {
   __shared__ __align__(16) SelectSmem s;
-  const SelJob j = B.job[blockIdx.x];
+  SelJob j = B.job[blockIdx.x];
+  grid_wait(j.plane);
   const float v = sel_finish(s, B.state + (size_t)blockIdx.x * SEL_HIST,
                              SelChan{j.plane, j.format, 1, B.H, B.W, B.pitch}, j.rank);
   if (threadIdx.x == 0) *j.out = v;
@@ -145,8 +151,9 @@ __global__ void __launch_bounds__(EXEC_THREADS) k_sel_finish(const __grid_consta
 
 // out = a (op) b pixel by pixel over H x W (row pitch `pitch` elements); b
 // is a plane or, when null, the constant c.  One IEEE rounding per pixel.
-__global__ void k_arith(int op, const void* __restrict__ a, int a_format, const void* b,
+__global__ void k_arith(int op, const void* a, int a_format, const void* b,
                         int b_format, float c, float* out, int H, int W, int pitch) {
+  grid_wait(a, b);
   const long long n = (long long)H * W;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x) {
@@ -172,6 +179,7 @@ __global__ void k_arith(int op, const void* __restrict__ a, int a_format, const 
 __global__ void __launch_bounds__(EXEC_THREADS, 2)
 k_ccl_local(const uint32_t* mask, const uint32_t* phi1, MaskGeom g, int tiles_x, int conn,
             CclScratch sc, int32_t* status) {
+  grid_wait();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   CclSmem& s = *reinterpret_cast<CclSmem*>(smem_raw);
   const CclGeom geo = ccl_geom(g.H, g.W, g.Wp, blockIdx.x, tiles_x, slice_rows(g), ccl_rows(g));
@@ -188,6 +196,7 @@ k_ccl_local(const uint32_t* mask, const uint32_t* phi1, MaskGeom g, int tiles_x,
 // glen: entries of G (H*W for labels, 2*H*W for rho keys).
 __global__ void k_ccl_merge(const uint32_t* mask, MaskGeom g, int tiles_x, int conn, int32_t* G,
                             int glen, int32_t* status) {
+  grid_wait();
   const int Hs = slice_rows(g);
   const int n = merge_units(g.H, g.Wp, tiles_x, Hs, ccl_rows(g));
   const int wpb = blockDim.x >> 5;
@@ -198,6 +207,7 @@ __global__ void k_ccl_merge(const uint32_t* mask, MaskGeom g, int tiles_x, int c
 __global__ void __launch_bounds__(EXEC_THREADS, 2)
 k_ccl_final_labels(const uint32_t* mask, MaskGeom g, int tiles_x, int conn, CclScratch sc,
                    int32_t* status) {
+  grid_wait();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   CclSmem& s = *reinterpret_cast<CclSmem*>(smem_raw);
   const CclGeom geo = ccl_geom(g.H, g.W, g.Wp, blockIdx.x, tiles_x, slice_rows(g), ccl_rows(g));
@@ -209,6 +219,7 @@ k_ccl_final_labels(const uint32_t* mask, MaskGeom g, int tiles_x, int conn, CclS
 __global__ void __launch_bounds__(EXEC_THREADS, 3)
 k_rz_final(const uint32_t* phi2, MaskGeom g, int tiles_x, int conn, CclScratch sc, uint32_t* Z,
            int32_t* status) {
+  grid_wait();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const CclGeom geo = ccl_geom(g.H, g.W, g.Wp, blockIdx.x, tiles_x, slice_rows(g), ccl_rows(g));
   rz_tile_select(*reinterpret_cast<RzSmem*>(smem_raw), phi2, geo, conn,
@@ -217,7 +228,7 @@ k_rz_final(const uint32_t* phi2, MaskGeom g, int tiles_x, int conn, CclScratch s
 
 // ----------------------------------------------------------- conversion --
 
-__global__ void k_pack_u8(const uint8_t* __restrict__ src, MaskGeom g, uint32_t* __restrict__ out) {
+__global__ void k_pack_u8(const uint8_t* src, MaskGeom g, uint32_t* out) {
   const int lane = threadIdx.x & 31;
   const long long nwords = (long long)g.H * g.Wp;
   const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
@@ -232,7 +243,7 @@ __global__ void k_pack_u8(const uint8_t* __restrict__ src, MaskGeom g, uint32_t*
   }
 }
 
-__global__ void k_unpack_u8(const uint32_t* __restrict__ src, MaskGeom g, uint8_t* __restrict__ out) {
+__global__ void k_unpack_u8(const uint32_t* src, MaskGeom g, uint8_t* out) {
   const long long n = (long long)g.H * g.W;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x) {
@@ -242,14 +253,11 @@ __global__ void k_unpack_u8(const uint32_t* __restrict__ src, MaskGeom g, uint8_
   }
 }
 
-// n vectors from src to dst.  Launched so that it may come up while the kernel
-// before it ends: it waits for that one's results, and then lets the next one
-// come up.
+// n vectors from src to dst.
 constexpr int COPY_UNR = 4;
-__global__ void __launch_bounds__(kThreads) k_copy(const uint4* __restrict__ src, uint4* __restrict__ dst,
+__global__ void __launch_bounds__(kThreads) k_copy(const uint4* src, uint4* dst,
                                                    unsigned n) {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  grid_wait();
   const unsigned first = blockIdx.x * (kThreads * COPY_UNR) + threadIdx.x;
   uint4 v[COPY_UNR];
 #pragma unroll
@@ -278,22 +286,20 @@ cudaError_t launch_thresholds(const void* plane, int format, MaskGeom g, const T
                               cudaStream_t st) {
   const int grid = grid_for((long long)g.H * g.Wp * 2, kThreads, 152 * 8);
   switch (n) {
-    case 1: k_thresholds<1><<<grid, kThreads, 0, st>>>(plane, format, g, T); break;
-    case 2: k_thresholds<2><<<grid, kThreads, 0, st>>>(plane, format, g, T); break;
-    case 3: k_thresholds<3><<<grid, kThreads, 0, st>>>(plane, format, g, T); break;
-    case THR_SET: k_thresholds<THR_SET><<<grid, kThreads, 0, st>>>(plane, format, g, T); break;
+    case 1: return launch_early(k_thresholds<1>, grid, kThreads, 0, st, plane, format, g, T);
+    case 2: return launch_early(k_thresholds<2>, grid, kThreads, 0, st, plane, format, g, T);
+    case 3: return launch_early(k_thresholds<3>, grid, kThreads, 0, st, plane, format, g, T);
+    case THR_SET: return launch_early(k_thresholds<THR_SET>, grid, kThreads, 0, st, plane, format, g, T);
     default: return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
 }
 
 template <int OP>
 static cudaError_t pointwise(const uint32_t* a, const uint32_t* b, MaskGeom g, uint32_t* out,
                              cudaStream_t st) {
-  k_pointwise<OP><<<grid_for((long long)g.H * (g.Wp >> 2), kThreads), kThreads, 0, st>>>(
-      reinterpret_cast<const uint4*>(a), reinterpret_cast<const uint4*>(b), g,
-      reinterpret_cast<uint4*>(out));
-  return cudaGetLastError();
+  return launch_early(k_pointwise<OP>, grid_for((long long)g.H * (g.Wp >> 2), kThreads), kThreads, 0,
+                      st, reinterpret_cast<const uint4*>(a), reinterpret_cast<const uint4*>(b), g,
+                      reinterpret_cast<uint4*>(out));
 }
 cudaError_t launch_not(const uint32_t* a, MaskGeom g, uint32_t* out, cudaStream_t st) {
   return pointwise<0>(a, nullptr, g, out, st);
@@ -315,9 +321,8 @@ cudaError_t launch_const(MaskGeom g, bool value, uint32_t* out, cudaStream_t st)
 }
 cudaError_t launch_near(const uint32_t* a, MaskGeom g, int conn, uint32_t* out,
                         cudaStream_t st) {
-  k_near<<<grid_for((long long)g.H * (g.Wp >> 2), kThreads), kThreads, 0, st>>>(
-      a, g, conn, reinterpret_cast<uint4*>(out));
-  return cudaGetLastError();
+  return launch_early(k_near, grid_for((long long)g.H * (g.Wp >> 2), kThreads), kThreads, 0, st, a, g,
+                      conn, reinterpret_cast<uint4*>(out));
 }
 
 size_t select_scratch_bytes(int n) {
@@ -343,20 +348,17 @@ cudaError_t launch_selects(const SelJob* jobs, int n, int H, int W, int pitch, v
     const dim3 grid(select_blocks((int64_t)H * W, m, 2 * 152), m);
     // (16-bit keys: two passes of 12 bits after one that missed)
     for (int pass = 0; pass < (wide ? SEL_PASSES : 3); ++pass) {
-      k_sel_pass<<<grid, EXEC_THREADS, 0, st>>>(B, pass);
-      if ((e = cudaGetLastError())) return e;
+      if ((e = launch_early(k_sel_pass, grid, EXEC_THREADS, 0, st, B, pass))) return e;
     }
-    k_sel_finish<<<m, EXEC_THREADS, 0, st>>>(B);
-    if ((e = cudaGetLastError())) return e;
+    if ((e = launch_early(k_sel_finish, m, EXEC_THREADS, 0, st, B))) return e;
   }
   return cudaSuccess;
 }
 
 cudaError_t launch_arith(int op, const void* a, int a_format, const void* b, int b_format, float c,
                          float* out, int H, int W, int pitch, cudaStream_t st) {
-  k_arith<<<grid_for((long long)H * W, kThreads), kThreads, 0, st>>>(op, a, a_format, b, b_format,
-                                                                    c, out, H, W, pitch);
-  return cudaGetLastError();
+  return launch_early(k_arith, grid_for((long long)H * W, kThreads), kThreads, 0, st, op, a, a_format, b,
+                      b_format, c, out, H, W, pitch);
 }
 
 int ccl_tiles_y(int H, int Hs, int cth) {
@@ -405,23 +407,35 @@ long long ccl_merge_units(int H, int Wp, int Hs, int cth) {
 }
 int ccl_tile_cap_host(int Wp, int cth) { return (cth / 2) * std::min(CCL_TWW, Wp) * 32; }
 
+// Labelling kernels come up early where their tiles are one wave (two blocks
+// an SM), and not in a captured graph: with more tiles the early blocks are in
+// the way of the waves still to come (8192 x 8192: 395 us early, 387 not), and
+// between the nodes of a graph there is less to hide (a chain of 75 selects at
+// 2048 x 2048: 2.85 ms early, 2.78 not).  On a stream of its own 3001 x 2777
+// labelling takes 49 us early and 51.5 not.
+static bool ccl_early(int tiles, cudaStream_t st) {
+  cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
+  return tiles <= 2 * 152 && cudaStreamIsCapturing(st, &s) == cudaSuccess &&
+         s == cudaStreamCaptureStatusNone;
+}
+
 cudaError_t launch_ccl_labels(const uint32_t* mask, MaskGeom g, int conn, CclScratch sc,
                               int32_t* status, cudaStream_t st) {
   cudaError_t e = ccl_set_attrs();
   if (e) return e;
   const int ty = ccl_tiles_y(g.H, g.Hs, ccl_rows(g)), tx = ccl_tiles_x(g.Wp);
   const size_t sm = sizeof(CclSmem);
+  const bool early = ccl_early(ty * tx, st);
   int32_t* labels = sc.G;
-  k_ccl_local<<<ty * tx, EXEC_THREADS, sm, st>>>(mask, nullptr, g, tx, conn, sc, status);
-  if ((e = cudaGetLastError())) return e;
+  e = launch_kernel(early, k_ccl_local, ty * tx, EXEC_THREADS, sm, st, mask, nullptr, g, tx, conn, sc, status);
+  if (e) return e;
   const long long nm = ccl_merge_units(g.H, g.Wp, g.Hs, ccl_rows(g)) * 32LL;
   if (nm > 0) {
-    k_ccl_merge<<<grid_for(nm, kThreads), kThreads, 0, st>>>(mask, g, tx, conn, labels,
-                                                             g.H * g.W, status);
-    if ((e = cudaGetLastError())) return e;
+    e = launch_kernel(early, k_ccl_merge, grid_for(nm, kThreads), kThreads, 0, st, mask, g, tx, conn, labels,
+                     g.H * g.W, status);
+    if (e) return e;
   }
-  k_ccl_final_labels<<<ty * tx, EXEC_THREADS, sm, st>>>(mask, g, tx, conn, sc, status);
-  return cudaGetLastError();
+  return launch_kernel(early, k_ccl_final_labels, ty * tx, EXEC_THREADS, sm, st, mask, g, tx, conn, sc, status);
 }
 
 cudaError_t launch_rz(const uint32_t* phi1, const uint32_t* phi2, MaskGeom g, int conn,
@@ -430,16 +444,17 @@ cudaError_t launch_rz(const uint32_t* phi1, const uint32_t* phi2, MaskGeom g, in
   if (e) return e;
   const int ty = ccl_tiles_y(g.H, g.Hs, ccl_rows(g)), tx = ccl_tiles_x(g.Wp);
   const size_t sm = sizeof(CclSmem);
-  k_ccl_local<<<ty * tx, EXEC_THREADS, sm, st>>>(phi2, phi1, g, tx, conn, sc, status);
-  if ((e = cudaGetLastError())) return e;
+  const bool early = ccl_early(ty * tx, st);
+  e = launch_kernel(early, k_ccl_local, ty * tx, EXEC_THREADS, sm, st, phi2, phi1, g, tx, conn, sc, status);
+  if (e) return e;
   const long long nm = ccl_merge_units(g.H, g.Wp, g.Hs, ccl_rows(g)) * 32LL;
   if (nm > 0) {
-    k_ccl_merge<<<grid_for(nm, kThreads), kThreads, 0, st>>>(phi2, g, tx, conn, sc.G,
-                                                             2 * g.H * g.W, status);
-    if ((e = cudaGetLastError())) return e;
+    e = launch_kernel(early, k_ccl_merge, grid_for(nm, kThreads), kThreads, 0, st, phi2, g, tx, conn, sc.G,
+                     2 * g.H * g.W, status);
+    if (e) return e;
   }
-  k_rz_final<<<ty * tx, EXEC_THREADS, sizeof(RzSmem), st>>>(phi2, g, tx, conn, sc, Z, status);
-  return cudaGetLastError();
+  return launch_kernel(early, k_rz_final, ty * tx, EXEC_THREADS, sizeof(RzSmem), st, phi2, g, tx, conn, sc, Z,
+                      status);
 }
 
 cudaError_t launch_pack_u8(const uint8_t* src, MaskGeom g, uint32_t* out, cudaStream_t st) {
@@ -455,17 +470,8 @@ cudaError_t launch_copy(const void* src, void* dst, size_t bytes, cudaStream_t s
   const size_t n = bytes / 16, per_block = (size_t)kThreads * COPY_UNR;
   if (bytes % 16 || n > 0x7FFFFFFFu) return cudaErrorInvalidValue;
   if (!n) return cudaSuccess;
-  cudaLaunchAttribute early{};
-  early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  early.val.programmaticStreamSerializationAllowed = 1;
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)((n + per_block - 1) / per_block));
-  cfg.blockDim = dim3(kThreads);
-  cfg.stream = st;
-  cfg.attrs = &early;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_copy, static_cast<const uint4*>(src), static_cast<uint4*>(dst),
-                            (unsigned)n);
+  return launch_early(k_copy, dim3((unsigned)((n + per_block - 1) / per_block)), kThreads, 0, st,
+                      static_cast<const uint4*>(src), static_cast<uint4*>(dst), (unsigned)n);
 }
 cudaError_t launch_clear_padding(uint32_t* m, MaskGeom g, cudaStream_t st) {
   k_clear_padding<<<grid_for((long long)g.H * g.Wp, kThreads * 4), kThreads, 0, st>>>(m, g);

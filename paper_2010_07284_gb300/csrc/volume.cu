@@ -19,6 +19,7 @@
 #include "dev_ccl.cuh"
 #include "dev_common.cuh"
 #include "kernels.h"
+#include "launch.cuh"
 
 namespace vl {
 
@@ -66,8 +67,9 @@ VL_DEV uint32_t near3_word(const uint32_t* a, const MaskGeom& g, int conn, int y
   return res & vmask(w, g.W);
 }
 
-__global__ void k_near3(const uint32_t* __restrict__ a, MaskGeom g, int conn,
-                        uint32_t* __restrict__ out) {
+__global__ void k_near3(const uint32_t* a, MaskGeom g, int conn,
+                        uint32_t* out) {
+  grid_wait(a);
   const long long nwords = (long long)g.H * g.Wp;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < nwords;
        i += (long long)gridDim.x * blockDim.x) {
@@ -123,6 +125,7 @@ VL_DEV uint32_t fill_down(uint32_t hit, uint32_t c) {
 // start of either row took 147 to 284 us on a 155 x 240 x 240 scan; this
 // takes 50 to 104.)
 __global__ void k_zmerge(const uint32_t* m, MaskGeom g, int conn, int32_t* L, int32_t* status) {
+  grid_wait(m);
   const int Hs = slice_rows(g), D = g.H / Hs;
   const int npx = g.H * g.W;
   const long long n = (long long)(D - 1) * Hs * g.Wp;
@@ -179,6 +182,7 @@ __global__ void k_zmerge(const uint32_t* m, MaskGeom g, int conn, int32_t* L, in
 // node only moves to an ancestor, and the root is the label of every node
 // on the way).
 __global__ void k_relabel(const uint32_t* m, MaskGeom g, int32_t* L, int32_t* status) {
+  grid_wait(m);
   const int npx = g.H * g.W;
   // grid-stride over the voxels, row and column stepped instead of divided
   const int stride = gridDim.x * blockDim.x;
@@ -202,6 +206,7 @@ __global__ void k_relabel(const uint32_t* m, MaskGeom g, int32_t* L, int32_t* st
 // voxels would be a pass over the volume for these few.
 __global__ void k_seed_flags(const uint32_t* phi1, const uint32_t* phi2, MaskGeom g, int conn,
                              int32_t* L, uint8_t* F, int32_t* status) {
+  grid_wait(phi1, phi2);
   const long long nwords = (long long)g.H * g.Wp;
   const int npx = g.H * g.W;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < nwords;
@@ -226,6 +231,7 @@ __global__ void k_seed_flags(const uint32_t* phi1, const uint32_t* phi2, MaskGeo
 // phi2 inside the word (a run is one component), the run's bits taken whole.
 __global__ void k_select_flagged(const uint32_t* phi2, MaskGeom g, int32_t* L, const uint8_t* F,
                                  uint32_t* Z, int32_t* status) {
+  grid_wait(phi2, F);
   const long long nwords = (long long)g.H * g.Wp;
   const int npx = g.H * g.W;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < nwords;
@@ -250,8 +256,8 @@ __global__ void k_select_flagged(const uint32_t* phi2, MaskGeom g, int32_t* L, c
 }  // namespace
 
 cudaError_t launch_near3(const uint32_t* a, MaskGeom g, int conn, uint32_t* out, cudaStream_t st) {
-  k_near3<<<grid_for((long long)g.H * g.Wp, kThreads), kThreads, 0, st>>>(a, g, conn, out);
-  return cudaGetLastError();
+  return launch_early(k_near3, grid_for((long long)g.H * g.Wp, kThreads), kThreads, 0, st, a, g, conn,
+                      out);
 }
 
 // The union-find of a volume's components: every voxel's key leads to its
@@ -263,30 +269,28 @@ static cudaError_t launch_components3(const uint32_t* mask, MaskGeom g, int conn
   const int Hs = slice_rows(g), D = g.H / Hs;
   if (D < 2) return cudaSuccess;
   const long long words = (long long)(D - 1) * Hs * g.Wp;
-  k_zmerge<<<grid_for(words, kThreads), kThreads, 0, st>>>(mask, g, conn, sc.G, status);
-  return cudaGetLastError();
+  return launch_early(k_zmerge, grid_for(words, kThreads), kThreads, 0, st, mask, g, conn, sc.G, status);
 }
 
 cudaError_t launch_labels3(const uint32_t* mask, MaskGeom g, int conn, CclScratch sc,
                            int32_t* status, cudaStream_t st) {
   cudaError_t e = launch_components3(mask, g, conn, sc, status, st);
   if (e || g.H == slice_rows(g)) return e;
-  k_relabel<<<grid_for((long long)g.H * g.W, kThreads * 4), kThreads, 0, st>>>(mask, g, sc.G, status);
-  return cudaGetLastError();
+  return launch_early(k_relabel, grid_for((long long)g.H * g.W, kThreads * 4), kThreads, 0, st, mask, g,
+                      sc.G, status);
 }
 
 cudaError_t launch_rz3(const uint32_t* phi1, const uint32_t* phi2, MaskGeom g, int conn,
                        Rz3Scratch sc, uint32_t* Z, int32_t* status, cudaStream_t st) {
-  cudaError_t e = launch_components3(phi2, g, conn, sc.ccl, status, st);
+  cudaError_t e = cudaMemsetAsync(sc.F, 0, (size_t)g.H * g.W, st);
+  if (!e) e = launch_components3(phi2, g, conn, sc.ccl, status, st);
   if (e) return e;
-  if ((e = cudaMemsetAsync(sc.F, 0, (size_t)g.H * g.W, st))) return e;
   const long long nwords = (long long)g.H * g.Wp;
-  k_seed_flags<<<grid_for(nwords, kThreads), kThreads, 0, st>>>(phi1, phi2, g, conn, sc.ccl.G, sc.F,
-                                                                status);
-  if ((e = cudaGetLastError())) return e;
-  k_select_flagged<<<grid_for(nwords, kThreads), kThreads, 0, st>>>(phi2, g, sc.ccl.G, sc.F, Z,
-                                                                    status);
-  return cudaGetLastError();
+  e = launch_early(k_seed_flags, grid_for(nwords, kThreads), kThreads, 0, st, phi1, phi2, g, conn,
+                   sc.ccl.G, sc.F, status);
+  if (e) return e;
+  return launch_early(k_select_flagged, grid_for(nwords, kThreads), kThreads, 0, st, phi2, g, sc.ccl.G,
+                      sc.F, Z, status);
 }
 
 }  // namespace vl
