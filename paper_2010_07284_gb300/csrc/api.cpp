@@ -427,7 +427,7 @@ vl_status batch_build(vl_context* ctx, const vl_job* jobs, int n_jobs, cudaStrea
           }
           case SK_RZ_FINAL: sub_us = 10.0 * J[j].cth / CCL_TH; break;
           case SK_RANK: sub_us = 50.0; break;
-          case SK_ARITH: sub_us = 10.0 + 2.0 * sd.insn_cnt; break;
+          case SK_ARITH: sub_us = 5.0 + 0.5 * sd.insn_cnt; break;
           // a select by one block: 10 us and 3 pixels a ns; a share of one
           case SK_PCT_PASS: sub_us = 10.0; break;
           default:
@@ -559,6 +559,7 @@ vl_status batch_build(vl_context* ctx, const vl_job* jobs, int n_jobs, cudaStrea
     d.images = reinterpret_cast<const DevImage*>(tb + I.off_images);
     d.arith = reinterpret_cast<const ArithInsn*>(tb + f_arith[I.formula_idx]);
     d.n_arith = (int32_t)P.arith.size();
+    d.arith_regs = P.arith_regs;
     d.first_num_image = n_own;
     uint32_t** hs = reinterpret_cast<uint32_t**>(&host[I.off_slotptrs]);
     const size_t mask_bytes = (size_t)I.H * I.Wp * 4;

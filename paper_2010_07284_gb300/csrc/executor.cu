@@ -106,42 +106,82 @@ VL_DEV void rank_rows(const float* tv, const RankTab& T, const void* plane, int 
   }
 }
 
-// Number terms of rows [sub * ARITH_ROWS, +ARITH_ROWS): the program runs per
-// pixel on a register file in shared memory (register q of thread t at
-// R[q * blockDim + t]; no local memory).
-VL_DEV void arith_rows(const DevJob& J, int sub, unsigned char* smem) {
-  const int nt = blockDim.x, n = J.n_arith;
-  float* R = reinterpret_cast<float*>(smem);
-  ArithInsn* prog = reinterpret_cast<ArithInsn*>(R + (size_t)kArithMaxRegs * nt);
-  for (int i = threadIdx.x; i < n; i += nt) prog[i] = J.arith[i];
-  __syncthreads();
-  float* r = R + threadIdx.x;
+// One operation, rounded once: the _rn intrinsics are never contracted into
+// fused multiply-adds.
+VL_DEV float arith_op(uint32_t op, float u, float w) {
+  switch (op) {
+    case A_ADD: return __fadd_rn(u, w);
+    case A_SUB: return __fsub_rn(u, w);
+    case A_MUL: return __fmul_rn(u, w);
+    default: return __fdiv_rn(u, w);
+  }
+}
+
+// Number terms of rows [sub * ARITH_ROWS, +ARITH_ROWS), for VECS vectors of
+// four pixels a thread at a time: instructions, with the images' addresses in
+// them, and the registers (q of vector u of thread t at R[(q * VECS + u) * nt +
+// t]) lie in shared memory; nt threads work.  Pixels behind a row's end are worked
+// out too: rows are 32 * Wp elements long.
+//
+// Bound by latency, of the loads and of one instruction after the other, so
+// as many vectors as the registers leave room for, and four rows an item, so
+// that an image of a thousand rows has items for most blocks.  (Nine
+// instructions on two 1021 x 1530 uint16 channels: 11.6 us; pixel by pixel, in
+// items of eight rows, 54.)
+constexpr int ARITH_PROG_BYTES = 16 * kArithMaxInsns;
+template <int VECS>
+VL_DEV void arith_rows(const DevJob& J, int sub, unsigned char* smem, int nt) {
+  const int n = J.n_arith;
+  uint4* prog = reinterpret_cast<uint4*>(smem);
+  float4* r = reinterpret_cast<float4*>(smem + ARITH_PROG_BYTES) + threadIdx.x;
   const size_t plane = (size_t)J.H * J.pitch;
-  const int y0 = sub * ARITH_ROWS, rows = min(J.H - y0, ARITH_ROWS);
-  for (int idx = threadIdx.x; idx < rows * J.W; idx += nt) {
-    const int y = y0 + idx / J.W, x = idx - (idx / J.W) * J.W;
-    const size_t off = (size_t)y * J.pitch + x;
+  for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    const ArithInsn A = J.arith[i];
+    uint4 w = make_uint4(A.op | A.dst << 8 | A.a << 16 | (uint32_t)A.b << 24, __float_as_uint(A.c), 0u, 0u);
+    if (A.op == A_VALUE || A.op == A_STORE) {
+      const DevImage im = J.images[A.op == A_VALUE ? A.img : J.first_num_image + A.img];
+      const unsigned long long p = (unsigned long long)chan_ptr(im, A.op == A_VALUE ? A.ch : 0, plane);
+      w.y = (im.format == PX_U16 ? 1u : 0u) | (im.written ? 2u : 0u);
+      w.z = (uint32_t)p;
+      w.w = (uint32_t)(p >> 32);
+    }
+    prog[i] = w;
+  }
+  __syncthreads();
+  const int y0 = sub * ARITH_ROWS, rows = min(J.H - y0, ARITH_ROWS), vpr = (J.W + 3) >> 2;
+  const int total = rows * vpr;
+  if ((int)threadIdx.x >= nt) return;
+  for (int first = threadIdx.x; first < total; first += nt * VECS) {
+    size_t off[VECS];
+#pragma unroll
+    for (int u = 0; u < VECS; ++u) {
+      const int idx = min(first + u * nt, total - 1);  // (the last vector again: the same values)
+      const int y = idx / vpr;
+      off[u] = (size_t)(y0 + y) * J.pitch + 4 * (idx - y * vpr);
+    }
     for (int k = 0; k < n; ++k) {
-      const ArithInsn A = prog[k];
-      if (A.op == A_VALUE) {
-        const DevImage im = J.images[A.img];
-        r[A.dst * nt] = ld_px(chan_ptr(im, A.ch, plane), im.format, !im.written, off);
-      } else if (A.op == A_STORE) {
-        float* out = static_cast<float*>(const_cast<void*>(J.images[J.first_num_image + A.img].data));
-        out[off] = r[A.a * nt];
+      const uint4 A = prog[k];
+      const uint32_t op = A.x & 0xFFu, dst = (A.x >> 8) & 0xFFu, a = (A.x >> 16) & 0xFFu, b = A.x >> 24;
+      void* p = reinterpret_cast<void*>((unsigned long long)A.z | (unsigned long long)A.w << 32);
+      if (op == A_VALUE) {
+        float4 v[VECS];
+#pragma unroll
+        for (int u = 0; u < VECS; ++u) v[u] = ld_px4(p, A.y & 1u ? PX_U16 : PX_F32, !(A.y & 2u), off[u]);
+#pragma unroll
+        for (int u = 0; u < VECS; ++u) r[(dst * VECS + u) * nt] = v[u];
+      } else if (op == A_STORE) {
+#pragma unroll
+        for (int u = 0; u < VECS; ++u)
+          *reinterpret_cast<float4*>(static_cast<float*>(p) + off[u]) = r[(a * VECS + u) * nt];
       } else {
-        const float u = r[A.a * nt];
-        const float w = A.b == kArithConst ? A.c : r[A.b * nt];
-        // one IEEE rounding per operation: the _rn intrinsics are never
-        // contracted into fused multiply-adds
-        float z;
-        switch (A.op) {
-          case A_ADD: z = __fadd_rn(u, w); break;
-          case A_SUB: z = __fsub_rn(u, w); break;
-          case A_MUL: z = __fmul_rn(u, w); break;
-          default: z = __fdiv_rn(u, w); break;
+        const float c = __uint_as_float(A.y);
+#pragma unroll
+        for (int u = 0; u < VECS; ++u) {
+          const float4 x = r[(a * VECS + u) * nt];
+          const float4 y = b == kArithConst ? make_float4(c, c, c, c) : r[(b * VECS + u) * nt];
+          r[(dst * VECS + u) * nt] = make_float4(arith_op(op, x.x, y.x), arith_op(op, x.y, y.y),
+                                                 arith_op(op, x.z, y.z), arith_op(op, x.w, y.w));
         }
-        r[A.dst * nt] = z;
       }
     }
   }
@@ -206,8 +246,12 @@ __device__ __noinline__ void rank_item(int sub) {
             J.planes + (size_t)T.plane0 * J.H * J.Wp);
 }
 
-__device__ __noinline__ void arith_item(int sub) {
-  arith_rows(s_job, sub, exec_smem);
+__device__ __noinline__ void arith_item(int sub, int smem_bytes) {
+  const int reg = 16 * EXEC_THREADS;  // bytes of a register, a vector each thread
+  const int room = (smem_bytes - ARITH_PROG_BYTES) / (reg * max(s_job.arith_regs, 1));
+  if (room >= 4) arith_rows<4>(s_job, sub, exec_smem, EXEC_THREADS);
+  else if (room >= 2) arith_rows<2>(s_job, sub, exec_smem, EXEC_THREADS);
+  else arith_rows<1>(s_job, sub, exec_smem, room ? EXEC_THREADS : EXEC_THREADS / 2);
 }
 
 __device__ __noinline__ void rz_local_item(int sub, int per_rz) {
@@ -260,7 +304,7 @@ VL_DEV void run_subitem(int sub, int per_rz, const ExecLaunch& L) {
     case SK_PCT_PASS: percentile_pass_item(sub); break;
     case SK_GROUP: group_item(sub, L); break;
     case SK_RANK: rank_item(sub); break;
-    case SK_ARITH: arith_item(sub); break;
+    case SK_ARITH: arith_item(sub, L.smem_bytes); break;
     case SK_RZ_LOCAL: rz_local_item(sub, per_rz); break;
     case SK_RZ_MERGE: rz_merge_item(sub, per_rz); break;
     case SK_RZ_FINAL: rz_final_item(sub, per_rz); break;
@@ -360,7 +404,7 @@ size_t exec_smem_bytes(int group_buffers, int group_rows, int tile_words) {
   size_t g = GROUP_PROG_BYTES + (size_t)group_buffers * group_buffer_bytes(group_rows, tile_words);
   size_t m = sizeof(CclSmem);
   if (sizeof(SelectSmem) > m) m = sizeof(SelectSmem);
-  const size_t arith = (size_t)kArithMaxRegs * EXEC_THREADS * 4 + sizeof(ArithInsn) * kArithMaxInsns;
+  const size_t arith = (size_t)kArithMaxRegs * (EXEC_THREADS / 2) * 16 + ARITH_PROG_BYTES;
   if (arith > m) m = arith;
   if (g > m) m = g;
   return (m + 15) & ~(size_t)15;

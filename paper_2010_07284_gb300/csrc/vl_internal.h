@@ -115,7 +115,7 @@ enum StepKind : int32_t {
 };
 
 // Rows of one arithmetic work item.
-constexpr int ARITH_ROWS = 8;
+constexpr int ARITH_ROWS = 4;
 
 // Number terms of a formula as one straight-line program run per pixel on a
 // register file of floats: A_VALUE loads image[img].channel[ch], the
@@ -253,7 +253,9 @@ struct DevJob {
   uint32_t* planes;             // rank-code planes, H x Wp words each
   const ArithInsn* arith;       // number-term program (SK_ARITH)
   int32_t n_arith;
+  int32_t arith_regs;           //   registers it uses
   int32_t first_num_image;      // image index of number image 0
+  int32_t pad_;
 };
 
 VL_HD_INLINE int32_t* rz_G(const DevJob& J, int k) {
