@@ -107,6 +107,56 @@ VL_DEV uint32_t fill_down(uint32_t hit, uint32_t c) {
   return t;
 }
 
+// The pairs of voxels (p, q) of word i of a slice and of the slice behind it
+// that have to be united, handed to f.
+template <class F>
+VL_DEV void zmerge_word(const uint32_t* m, const MaskGeom& g, int conn, long long i, F f) {
+  const int Hs = slice_rows(g);
+  int row, w, z, yz;
+  split_index(i, g.Wp, row, w);
+  split_index(row, Hs, z, yz);
+  const SliceRows R(m, g, w);
+  const uint32_t a = R.at(z, yz, 0);
+  if (!a) return;
+  const int p0 = row * g.W + 32 * w, q0 = p0 + Hs * g.W;  // first voxels of the words
+  auto unite = [&](uint32_t set, int dq) {
+    while (set) {
+      const int b = __ffs(set) - 1;
+      set &= set - 1;
+      f(p0 + b, q0 + b + dq);
+    }
+  };
+  const uint32_t b0 = R.at(z + 1, yz, 0), c = a & b0;
+  const uint32_t al = R.at(z, yz, -1), bl = R.at(z + 1, yz, -1);
+  const uint32_t au = R.at(z, yz - 1, 0), bu = R.at(z + 1, yz - 1, 0);
+  uint32_t cu = au & bu;  // contacts of the row above
+  if (conn == 26) cu |= (cu << 1) | (cu >> 1);
+  const uint32_t starts = c & ~((c << 1) | ((al & bl) >> 31));
+  unite(starts & ~fill_down(cu, c), 0);
+  if (conn != 26) return;
+  const uint32_t p = a & ~b0;
+  if (!p) return;
+  const uint32_t ar = R.at(z, yz, 1), br = R.at(z + 1, yz, 1);
+  // same row, one column apart
+  const uint32_t q = b0 & ~a;
+  unite(p & ((q << 1) | ((bl & ~al) >> 31)), -1);
+  unite(p & ((q >> 1) | ((br & ~ar) << 31)), 1);
+  const uint32_t a_left = (a << 1) | (al >> 31), a_right = (a >> 1) | (ar << 31);
+#pragma unroll
+  for (int dy = -1; dy <= 1; dy += 2) {
+    const uint32_t ay = dy < 0 ? au : R.at(z, yz + 1, 0), by = dy < 0 ? bu : R.at(z + 1, yz + 1, 0);
+    const uint32_t qy = by & ~ay;
+    const uint32_t over = p & qy;
+    unite(over & ~(over << 1), dy * g.W);
+    const uint32_t free = p & ~by;
+    if (!free) continue;
+    const uint32_t qyl = R.at(z + 1, yz + dy, -1) & ~R.at(z, yz + dy, -1);
+    const uint32_t qyr = R.at(z + 1, yz + dy, 1) & ~R.at(z, yz + dy, 1);
+    unite(free & ~a_left & ((qy << 1) | (qyl >> 31)), dy * g.W - 1);
+    unite(free & ~a_right & ((qy >> 1) | (qyr << 31)), dy * g.W + 1);
+  }
+}
+
 // Unite the components of slices z and z + 1; one thread per word of slice z.
 // L holds, for every voxel of the mask, its slice component's key (after the
 // 2D pass: the component's minimum index, which is a root).
@@ -123,58 +173,39 @@ VL_DEV uint32_t fill_down(uint32_t hit, uint32_t c) {
 // (else that one makes a pair one column closer), and of neighbouring pairs
 // in the same direction the first.  (A warp per row that offered every run
 // start of either row took 147 to 284 us on a 155 x 240 x 240 scan; this
-// takes 50 to 104.)
-__global__ void k_zmerge(const uint32_t* m, MaskGeom g, int conn, int32_t* L, int32_t* status) {
+// takes 16 to 51.)
+//
+// Pairs go to a list of the block's and are dealt out to its threads from
+// there: a thread that united those of its own word kept the others waiting
+// where the mask is dense (48 to 116 us).
+constexpr int ZMERGE_LIST = 3072;
+__global__ void __launch_bounds__(kThreads) k_zmerge(const uint32_t* m, MaskGeom g, int conn, int32_t* L,
+                                                     int32_t* status) {
+  __shared__ int2 list[ZMERGE_LIST];
+  __shared__ int listed;
   grid_wait(m);
   const int Hs = slice_rows(g), D = g.H / Hs;
   const int npx = g.H * g.W;
   const long long n = (long long)(D - 1) * Hs * g.Wp;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (long long)gridDim.x * blockDim.x) {
-    int row, w, z, yz;
-    split_index(i, g.Wp, row, w);
-    split_index(row, Hs, z, yz);
-    const SliceRows R(m, g, w);
-    const uint32_t a = R.at(z, yz, 0);
-    if (!a) continue;
-    const int p0 = row * g.W + 32 * w, q0 = p0 + Hs * g.W;  // first voxels of the words
-    auto unite = [&](uint32_t set, int dq) {
-      while (set) {
-        const int b = __ffs(set) - 1;
-        set &= set - 1;
-        const int ka = ldcg(&L[p0 + b]), kb = ldcg(&L[q0 + b + dq]);
-        if (ka != kb) g_union(L, ka, kb, npx, status);
-      }
-    };
-    const uint32_t b0 = R.at(z + 1, yz, 0), c = a & b0;
-    const uint32_t al = R.at(z, yz, -1), bl = R.at(z + 1, yz, -1);
-    const uint32_t au = R.at(z, yz - 1, 0), bu = R.at(z + 1, yz - 1, 0);
-    uint32_t cu = au & bu;  // contacts of the row above
-    if (conn == 26) cu |= (cu << 1) | (cu >> 1);
-    const uint32_t starts = c & ~((c << 1) | ((al & bl) >> 31));
-    unite(starts & ~fill_down(cu, c), 0);
-    if (conn != 26) continue;
-    const uint32_t p = a & ~b0;
-    if (!p) continue;
-    const uint32_t ar = R.at(z, yz, 1), br = R.at(z + 1, yz, 1);
-    // same row, one column apart
-    const uint32_t q = b0 & ~a;
-    unite(p & ((q << 1) | ((bl & ~al) >> 31)), -1);
-    unite(p & ((q >> 1) | ((br & ~ar) << 31)), 1);
-    const uint32_t a_left = (a << 1) | (al >> 31), a_right = (a >> 1) | (ar << 31);
-#pragma unroll
-    for (int dy = -1; dy <= 1; dy += 2) {
-      const uint32_t ay = dy < 0 ? au : R.at(z, yz + 1, 0), by = dy < 0 ? bu : R.at(z + 1, yz + 1, 0);
-      const uint32_t qy = by & ~ay;
-      const uint32_t over = p & qy;
-      unite(over & ~(over << 1), dy * g.W);
-      const uint32_t free = p & ~by;
-      if (!free) continue;
-      const uint32_t qyl = R.at(z + 1, yz + dy, -1) & ~R.at(z, yz + dy, -1);
-      const uint32_t qyr = R.at(z + 1, yz + dy, 1) & ~R.at(z, yz + dy, 1);
-      unite(free & ~a_left & ((qy << 1) | (qyl >> 31)), dy * g.W - 1);
-      unite(free & ~a_right & ((qy >> 1) | (qyr << 31)), dy * g.W + 1);
-    }
+  auto pair = [&](int p, int q) {
+    const int ka = ldcg(&L[p]), kb = ldcg(&L[q]);
+    if (ka != kb) g_union(L, ka, kb, npx, status);
+  };
+  for (long long base = (long long)blockIdx.x * blockDim.x; base < n;
+       base += (long long)gridDim.x * blockDim.x) {
+    if (threadIdx.x == 0) listed = 0;
+    __syncthreads();
+    const long long i = base + threadIdx.x;
+    if (i < n)
+      zmerge_word(m, g, conn, i, [&](int p, int q) {
+        const int at = atomicAdd(&listed, 1);
+        if (at < ZMERGE_LIST) list[at] = make_int2(p, q);
+        else pair(p, q);
+      });
+    __syncthreads();
+    const int k = min(listed, ZMERGE_LIST);
+    for (int j = threadIdx.x; j < k; j += blockDim.x) pair(list[j].x, list[j].y);
+    __syncthreads();
   }
 }
 
