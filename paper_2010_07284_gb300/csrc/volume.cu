@@ -67,15 +67,48 @@ VL_DEV uint32_t near3_word(const uint32_t* a, const MaskGeom& g, int conn, int y
   return res & vmask(w, g.W);
 }
 
-__global__ void k_near3(const uint32_t* a, MaskGeom g, int conn,
-                        uint32_t* out) {
+// N a on whole vectors of four words, one a thread: nine vector loads and the
+// words beside them instead of 27 loads a word.
+__global__ void __launch_bounds__(kThreads) k_near3(const uint32_t* a, MaskGeom g, int conn, uint4* out) {
   grid_wait(a);
-  const long long nwords = (long long)g.H * g.Wp;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < nwords;
+  const int nv = g.Wp >> 2, Hs = slice_rows(g), D = g.H / Hs;
+  const long long n = (long long)g.H * nv;
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x) {
-    int y, w;
-    split_index(i, g.Wp, y, w);
-    out[i] = near3_word(a, g, conn, y, w);
+    int y, jv, z, yz;
+    split_index(i, nv, y, jv);
+    split_index(y, Hs, z, yz);
+    const bool left = jv > 0, right = jv + 1 < nv;
+    const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+    // row (dy, dz) away, and the words beside its vector
+    auto inside = [&](int dy, int dz) {
+      return z + dz >= 0 && z + dz < D && yz + dy >= 0 && yz + dy < Hs;
+    };
+    auto at = [&](int dy, int dz) { return a + 4 * i + (long long)(dz * Hs + dy) * g.Wp; };
+    uint4 x = zero, o = zero;
+    uint32_t l = 0, e = 0;
+    if (conn == 26) {
+#pragma unroll
+      for (int dz = -1; dz <= 1; ++dz)
+#pragma unroll
+        for (int dy = -1; dy <= 1; ++dy)
+          if (inside(dy, dz)) {
+            const uint32_t* p = at(dy, dz);
+            x = or4(x, __ldg(reinterpret_cast<const uint4*>(p)));
+            if (left) l |= __ldg(p - 1);
+            if (right) e |= __ldg(p + 4);
+          }
+    } else {
+      const uint32_t* p = at(0, 0);
+      x = __ldg(reinterpret_cast<const uint4*>(p));
+      if (left) l = __ldg(p - 1);
+      if (right) e = __ldg(p + 4);
+      if (inside(-1, 0)) o = or4(o, __ldg(reinterpret_cast<const uint4*>(at(-1, 0))));
+      if (inside(1, 0)) o = or4(o, __ldg(reinterpret_cast<const uint4*>(at(1, 0))));
+      if (inside(0, -1)) o = or4(o, __ldg(reinterpret_cast<const uint4*>(at(0, -1))));
+      if (inside(0, 1)) o = or4(o, __ldg(reinterpret_cast<const uint4*>(at(0, 1))));
+    }
+    out[i] = clip_vec(near_vec(x, o, l, e), jv, g.W);
   }
 }
 
@@ -330,8 +363,8 @@ __global__ void __launch_bounds__(kThreads) k_select_flagged(const uint32_t* phi
 }  // namespace
 
 cudaError_t launch_near3(const uint32_t* a, MaskGeom g, int conn, uint32_t* out, cudaStream_t st) {
-  return launch_early(k_near3, grid_for((long long)g.H * g.Wp, kThreads), kThreads, 0, st, a, g, conn,
-                      out);
+  return launch_early(k_near3, grid_for((long long)g.H * (g.Wp >> 2), kThreads), kThreads, 0, st, a, g,
+                      conn, reinterpret_cast<uint4*>(out));
 }
 
 // The union-find of a volume's components: every voxel's key leads to its
