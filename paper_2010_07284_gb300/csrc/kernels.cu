@@ -414,9 +414,11 @@ int ccl_tile_cap_host(int Wp, int cth) { return (cth / 2) * std::min(CCL_TWW, Wp
 // 2048 x 2048: 2.85 ms early, 2.78 not).  On a stream of its own 3001 x 2777
 // labelling takes 49 us early and 51.5 not.
 static bool ccl_early(int tiles, cudaStream_t st) {
+  if (tiles > 2 * 152) return false;
   cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
-  return tiles <= 2 * 152 && cudaStreamIsCapturing(st, &s) == cudaSuccess &&
-         s == cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &s) == cudaSuccess) return s == cudaStreamCaptureStatusNone;
+  cudaGetLastError();  // (the legacy stream beside another one's capture; the launch says so)
+  return false;
 }
 
 cudaError_t launch_ccl_labels(const uint32_t* mask, MaskGeom g, int conn, CclScratch sc,
