@@ -24,9 +24,10 @@
 //
 // What bounds a select is instructions and the loads in front of them: a
 // block alone on its SM reads 3 pixels a ns, and has about 10 us of sample,
-// sort and histograms of its list to do besides.  Five selects of a 2048 x
-// 2048 float image over the whole grid: 41 us for the pass that counts, 18 us
-// (4.7 TB/s) for the one after it.  The three passes of one block per select
+// sort and histograms of its list to do besides.  Five selects of the four
+// float channels of a 155 x 240 x 240 scan over the whole grid: 60 us for the
+// pass that counts (70 with the ends of the range counted behind a branch),
+// 34 us (5.2 TB/s, partly from L2) for the one after it.  The three passes of one block per select
 // that histogrammed every pixel's digits before took 1.82 ms for three
 // 1021 x 1530 channels where this takes 35 us, and 124 us for a 240 x 240 one
 // (two blocks on an SM) where this takes 40; bound by atomics on shared
@@ -264,23 +265,19 @@ template <class F>
 VL_DEV void sel_count(SelectSmem& s, SelChan c, const SelRange& r, unsigned v0, unsigned v1,
                       F between) {
   uint32_t lt = 0, at_lo = 0, at_hi = 0, in = 0;
-  const uint32_t span = r.hi - r.lo;
+  // key - lo: below it wraps around, 0 and span are the ends, and one less is
+  // below span - 1 between them
+  const uint32_t span = r.hi - r.lo, inner = span ? span - 1u : 0u;
   sel_scan(c, v0, v1, [&](const uint32_t (&k)[SEL_KEYS]) {
-    uint32_t m = 0, h = 0;  // keys in the range, and those at its ends
+    uint32_t m = 0;
 #pragma unroll
     for (int q = 0; q < SEL_KEYS; ++q) {
+      const uint32_t d = k[q] - r.lo;
       lt += k[q] < r.lo;
-      if (k[q] - r.lo <= span) m |= 1u << q;
+      at_lo += d == 0;
+      at_hi += d == span;
+      if (d - 1u < inner) m |= 1u << q;
     }
-#pragma unroll
-    for (int q = 0; q < SEL_KEYS; ++q)
-      if ((m >> q) & 1u) {
-        const bool lo = k[q] == r.lo, hi = k[q] == r.hi;
-        at_lo += lo;
-        at_hi += hi;
-        if (lo || hi) h |= 1u << q;
-      }
-    m &= ~h;
     in += __popc(m);
     between(k, m);
   });
