@@ -6,8 +6,8 @@
 // iterated pointer jumping with host-checked termination, Sec. 3.3):
 //   1. tile-local: one CTA labels a tile of CCL_TH rows x CCL_TWW words.
 //      The union-find elements are the connected pieces of two-row strips,
-//      found with bit operations on the packed words; strips are united in
-//      shared memory with atomicMin along a binary tree of strip boundaries.
+//      found with bit operations on the packed words; they are united in
+//      shared memory with atomicMin, over all strip boundaries at once.
 //   2. publish: every foreground pixel on the tile border, and every local
 //      root that reaches the border, gets an entry G[gid] in a global
 //      union-find array indexed by linear pixel id gid = y*W + x.
@@ -267,9 +267,7 @@ VL_DEV void g_union(int32_t* G, int a, int b, int npx, int32_t* status) {
 // set columns always touch, diagonally at least); under 4-adjacency they are
 // those runs cut where the set row switches from A-only to B-only (or back)
 // between two columns.  These "strip runs" are the union-find elements.
-// Strips are then merged across the CCL_NS - 1 strip boundaries in a
-// binary-tree order (boundary b at level = trailing ones of b, plus one), so
-// every level unites disjoint groups of strips and the trees stay shallow.
+// Strips are then merged across the CCL_NS - 1 strip boundaries.
 // Across a boundary (rows A' = last row of the upper strip, B' = first row of
 // the lower one), the same two-row rule holds: every set pixel of A' and B'
 // inside one run of A' | B' (cut the same way for 4-adjacency) is connected,

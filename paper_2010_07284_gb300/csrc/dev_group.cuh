@@ -2,14 +2,14 @@
 //
 // A group is a sub-DAG of threshold atoms, not/and/or and N (Sec. 2) whose
 // inputs are image channels or masks materialised by earlier steps.  Every
-// value lives in a shared-memory buffer of (th + 2*halo) rows x (tww + 2)
-// words: the core tile plus `halo` rows above and below and one 32-px word
-// left and right.  A node whose value is needed `h` pixels beyond the core
+// value lives in a shared-memory buffer of (th + 2*halo) rows: the core tile
+// plus `halo` rows above and below and one vector of four 32-px words left and
+// right (of which the word next to the core counts).  A node whose value is needed `h` pixels beyond the core
 // is computed over rows [halo - h, halo + th + h); N consumes one pixel of
 // halo, so a chain of k N operators inside a group needs halo >= k (the
 // compiler caps it at 31, inside the one-word horizontal margin).  Pixels
-// outside the image are stored as 0, which is exactly the clipping of the
-// neighbourhood at the image border.
+// outside the image are stored as 0 where a neighbour may read them, which is
+// exactly the clipping of the neighbourhood at the image border.
 #pragma once
 #include "dev_common.cuh"
 

@@ -60,8 +60,8 @@ constexpr int RS_SUNION = 6 << 8;    // shared union-find ran past its bound
 constexpr int RS_GRANGE = 7 << 8;    // global union-find entry outside the image
 
 // --------------------------------------------------------- group bytecode
-// One instruction of a fused tile group.  Buffers are shared-memory tiles
-// of (th + 2*halo) rows x (tww + 2) words; `h` is the halo (in rows and
+// One instruction of a fused tile group.  Buffers are shared-memory tiles of
+// (th + 2*halo) rows x group_vecs vectors; `h` is the halo (in rows and
 // pixels) over which this node's value is needed.
 enum InsnOp : uint8_t {
   I_NOP = 0,
