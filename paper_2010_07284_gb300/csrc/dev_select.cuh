@@ -35,23 +35,14 @@
 // out.
 #pragma once
 #include "dev_common.cuh"
+#include "select_range.h"
 
 namespace vl {
 
 VL_DEV int sel_shift(int d) { return d == 0 ? 20 : d == 1 ? 8 : 0; }
 VL_DEV int sel_bins(int d) { return d == 2 ? 256 : SEL_BINS; }
 
-// Key of a float's bits: ordered like the float, -infinity at 0 and every NaN
-// above +infinity (the negative ones, whose bits sort below -infinity, wrap
-// around to the top).
-VL_DEV uint32_t sel_key(uint32_t u) {
-  return (u ^ ((uint32_t)((int32_t)u >> 31) | 0x80000000u)) - 0x007FFFFFu;
-}
-VL_DEV float sel_float(uint32_t key) {
-  const uint32_t k = key + 0x007FFFFFu;
-  return __uint_as_float((k & 0x80000000u) ? k ^ 0x80000000u : ~k);
-}
-constexpr uint32_t SEL_TOP_BITS = 0xFF800001u;  // the float bits of the highest key
+VL_DEV float sel_float(uint32_t key) { return __uint_as_float(sel_key_bits(key)); }
 
 constexpr int SEL_SAMPLE = 1024;
 struct SelectSmem {
@@ -178,23 +169,6 @@ VL_DEV void sel_pick(SelectSmem& s, const uint32_t* h, bool global, unsigned lon
   __syncthreads();
 }
 
-// Keys [lo, hi] among which the wanted one has rank `rank`.
-struct SelRange {
-  uint32_t lo, hi;
-  unsigned long long rank;
-  VL_DEV bool done() const { return lo == hi; }
-  // bits of key - lo below a bin
-  VL_DEV int shift() const { return max(0, 20 - __clz(hi - lo)); }
-  VL_DEV uint32_t bin(uint32_t key) const { return (key - lo) >> shift(); }
-  VL_DEV bool holds(uint32_t key) const { return key - lo <= hi - lo; }
-  VL_DEV void take(const SelectSmem& s) {  // the bin that was picked
-    const int sh = shift();
-    lo += s.digit << sh;
-    hi = min(hi, lo + ((1u << sh) - 1u));
-    rank -= s.below;
-  }
-};
-
 // Two keys that most likely enclose the key of rank k: order statistics of a
 // sample, 3.5 standard deviations of its rank to either side; the ends of the
 // key range where the sample ends, or where it would not be worth its sort.
@@ -241,23 +215,6 @@ VL_DEV SelRange sel_sample(SelectSmem& s, SelChan c, long long k) {
   return r;
 }
 
-// The range that the counts below, at and between the sample's keys leave for
-// rank k of the channel.  `between`: it is the one between them.
-VL_DEV SelRange sel_resolve(const SelRange& r, uint32_t top, const uint32_t* count, long long k,
-                            bool& between) {
-  unsigned long long rank = (unsigned long long)k;
-  between = false;
-  if (rank < count[0]) return SelRange{0u, r.lo - 1u, rank};
-  rank -= count[0];
-  if (rank < count[1]) return SelRange{r.lo, r.lo, rank};
-  rank -= count[1];
-  between = rank < count[3];
-  if (between) return SelRange{r.lo + 1u, r.hi - 1u, rank};
-  rank -= count[3];
-  if (rank < count[2]) return SelRange{r.hi, r.hi, rank};
-  return SelRange{r.hi + 1u, top, rank - count[2]};
-}
-
 // Counts of the sample's keys over vectors [v0, v1) into s.count, and
 // between(keys, which) for the keys between them (whole warps).  (Keys at r.lo
 // are not counted at r.hi again where the two are the same.)
@@ -300,8 +257,8 @@ VL_DEV void sel_clear(SelectSmem& s) {
 
 // One block selects rank k of the channel.  list: room for `cap` keys in
 // shared memory.  Returns the value in every thread (after a block barrier).
-VL_DEV float select_rank(SelectSmem& s, uint32_t* list, int cap,
-                                                 SelChan c, long long k) {
+VL_DEV float select_rank(SelectSmem& s, uint32_t* list, int cap, SelChan c, long long k,
+                         int32_t* status) {
   const unsigned n = c.vecs();
   const int lane = threadIdx.x & 31;
   const SelRange guess = sel_sample(s, c, k);
@@ -333,7 +290,7 @@ VL_DEV float select_rank(SelectSmem& s, uint32_t* list, int cap,
   SelRange r = sel_resolve(guess, c.top(), s.count, k, between);
   const uint32_t listed = s.count[3];
   const bool from_list = between && listed <= (uint32_t)cap;
-  while (!r.done()) {  // (at most three times: 12 bits of the range each)
+  for (int round = 0; round < SEL_ROUNDS && !r.done(); ++round) {
     sel_clear(s);
     __syncthreads();
     if (from_list) {
@@ -348,8 +305,9 @@ VL_DEV float select_rank(SelectSmem& s, uint32_t* list, int cap,
     }
     __syncthreads();
     sel_pick(s, s.hist, false, r.rank);
-    r.take(s);
+    r.take(s.digit, s.below);
   }
+  if (!r.done() && threadIdx.x == 0) set_status(status, ST_INTERNAL | RS_SELECT);
   __syncthreads();
   return c.value(r.lo);
 }
@@ -379,7 +337,7 @@ VL_DEV SelRange sel_range(SelectSmem& s, uint32_t* g, SelChan c, int passes, lon
   SelRange r = sel_resolve(SelRange{a.x, a.y, 0ull}, c.top(), count, k, between);
   for (int p = between ? 0 : 1; p < passes && !r.done(); ++p) {
     sel_pick(s, sel_hist_of(g, p), true, r.rank);
-    r.take(s);
+    r.take(s.digit, s.below);
   }
   return r;
 }

@@ -215,7 +215,7 @@ __device__ __noinline__ void percentile_item(int sub, int smem_bytes) {
   const float v =
       J.sel_hist ? sel_finish(s, J.sel_hist + (size_t)sub * SEL_HIST, c, select_rank_of(J, d))
                  : select_rank(s, reinterpret_cast<uint32_t*>(exec_smem + sizeof(SelectSmem)),
-                               (smem_bytes - (int)sizeof(SelectSmem)) / 4, c, select_rank_of(J, d));
+                               (smem_bytes - (int)sizeof(SelectSmem)) / 4, c, select_rank_of(J, d), J.status);
   if (threadIdx.x == 0) J.pct_val[d.slot] = v;
 }
 __device__ __noinline__ void percentile_pass_item(int sub) {

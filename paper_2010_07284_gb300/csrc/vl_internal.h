@@ -58,6 +58,7 @@ constexpr int RS_TLOAD = 4 << 8;     // saved tile state out of range
 constexpr int RS_TRUNS = 5 << 8;     // more strip runs than a tile holds
 constexpr int RS_SUNION = 6 << 8;    // shared union-find ran past its bound
 constexpr int RS_GRANGE = 7 << 8;    // global union-find entry outside the image
+constexpr int RS_SELECT = 8 << 8;    // percentile select not down to one key
 
 // --------------------------------------------------------- group bytecode
 // One instruction of a fused tile group.  Buffers are shared-memory tiles of
