@@ -93,8 +93,12 @@ typedef struct {
                              exercise the timeout path) */
   int64_t memory_budget;  /* bytes the server may hold; 0 = free HBM minus
                              a reserve */
-  int32_t tile_rows;      /* 0 = autotune; else rows per fused tile */
-  int32_t tile_words;     /* 0 = autotune; else 32-px words per fused tile */
+  int32_t tile_rows;      /* 0 = autotune; else rows per fused tile (<= 1024) */
+  int32_t tile_words;     /* 0 = autotune; else 32-px words per fused tile
+                             (<= 256).  VL_ERR_ARG when four buffers of
+                             tile_rows + 16 rows of tile_words words, rounded up
+                             to whole fours, and eight more do not fit one
+                             CTA's shared memory (227 KB on sm_103a) */
   int32_t reserved[6];
 } vl_config;
 

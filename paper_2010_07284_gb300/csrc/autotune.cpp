@@ -15,6 +15,7 @@
 #include <iterator>
 #include <set>
 
+#include "kernels.h"
 #include "runtime.h"
 
 namespace vl {
@@ -80,7 +81,8 @@ vl_tile_choice to_choice(const vl_context* ctx, const TileShape& t, int status, 
   c.tile_rows = t.per_op ? 0 : t.rows;
   c.tile_words = t.per_op ? 0 : t.words;
   c.ctas_per_sm = t.per_op ? 0
-                  : t.ctas_per_sm > 0 ? std::min(t.ctas_per_sm, ctx->ctas_per_sm) : ctx->ctas_per_sm;
+                  : t.ctas_per_sm > 0 ? std::min(t.ctas_per_sm, tile_shape_ctas(ctx, t))
+                                      : tile_shape_ctas(ctx, t);
   c.status = status;
   c.ms = ms;
   return c;
@@ -98,11 +100,26 @@ uint64_t plan_hash(const Plan& P) {
   return h;
 }
 
+size_t tile_shape_smem(const vl_context* ctx, const TileShape& t) {
+  return std::max(ctx->exec_smem, exec_smem_bytes(ctx->nb, t.rows + 2 * ctx->hmax, t.words));
+}
 bool tile_shape_fits(const vl_context* ctx, const TileShape& t) {
-  if (t.rows < 1 || t.words < 1) return false;
-  const int64_t bytes =
-      GROUP_PROG_BYTES + ctx->nb * group_buffer_bytes(t.rows + 2 * ctx->hmax, t.words);
-  return bytes <= (int64_t)ctx->exec_smem;
+  return t.rows >= 1 && t.words >= 1 && tile_shape_smem(ctx, t) <= ctx->exec_smem_max;
+}
+// (exec_smem is what two CTAs of an SM can have, or more)
+int tile_shape_ctas(const vl_context* ctx, const TileShape& t) {
+  return tile_shape_smem(ctx, t) > ctx->exec_smem ? 1 : ctx->ctas_per_sm;
+}
+
+// Shapes that a tile table may name and the autotuner tries: the tile's words
+// with one beside them on either side, for every buffer of a plan, in half an
+// SM's shared memory.  A measure of its own, so that which tables load does
+// not depend on how the buffers are laid out; a shape whose buffers then do
+// not fit (a tall tile of a few words) is passed over when a batch is built.
+constexpr int64_t kTableSmem = 115456;
+static bool tile_shape_in_table(const vl_context* ctx, const TileShape& t) {
+  return t.rows >= 1 && t.words >= 1 &&
+         (int64_t)ctx->nb * (t.rows + 2 * ctx->hmax) * (t.words + 2) * 4 <= kTableSmem;
 }
 
 TileShape pick_tile_shape(vl_context* ctx, const vl_job* jobs, int n_jobs, int* tuned,
@@ -197,8 +214,9 @@ extern "C" VL_API vl_status vl_autotune(vl_context* ctx, const vl_job* jobs, int
   }
   std::vector<TileShape> cands;
   for (const TileShape& base : bases) {
-    if (!tile_shape_fits(ctx, base)) continue;
+    if (!tile_shape_in_table(ctx, base) || !tile_shape_fits(ctx, base)) continue;
     for (int cps : cps_list) {
+      if (cps > tile_shape_ctas(ctx, base)) continue;
       TileShape t = base;
       t.ctas_per_sm = cps;
       cands.push_back(t);
@@ -314,7 +332,7 @@ extern "C" VL_API vl_status vl_tune_load(vl_context* ctx, const char* path) {
     if (r == 0 && w == 0 && c == 0) {
       t = TileShape{};
       t.per_op = true;
-    } else if (r < 1 || w < 1 || c < 0 || !tile_shape_fits(ctx, t)) {
+    } else if (c < 0 || !tile_shape_in_table(ctx, t)) {
       std::fclose(fh);
       return set_err(ctx, VL_ERR_ARG, "tile table entry does not fit this context");
     }
