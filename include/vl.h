@@ -484,7 +484,7 @@ VL_API vl_status vl_batch_result(vl_batch* b, int32_t job, vl_result** out);
 
 /* Step timeline of the last run of a batch made by a context with `trace`
  * set: for every (job, step) seven int64 values {job, step, kind, start_ns,
- * end_ns, busy_ns, wait_ns} -- kind as in vl_plan_step, start/end from the
+ * end_ns, busy_ns, wait_ns} -- steps and kinds as in vl_formula_plan, start/end from the
  * device global timer, busy = summed time of its work items, wait = summed
  * time its items spent waiting for the previous step.  Waits for the batch's
  * work.  Writes up to max_entries entries; *n_entries gets the total. */

@@ -198,10 +198,13 @@ int ccl_merge_chunks(int H, int Wp, int cth) {
 struct DevSteps {
   std::vector<StepDesc> steps;
   std::vector<int32_t> dep_off, deps;
+  std::vector<int32_t> at;  // of each step of the plan: its last one here (those
+                            // of a step follow one another)
 };
 DevSteps device_steps(const Plan& P, bool split_selects) {
   DevSteps D;
-  std::vector<int32_t> at(P.steps.size());
+  std::vector<int32_t>& at = D.at;
+  at.resize(P.steps.size());
   D.dep_off.push_back(0);
   for (size_t i = 0; i < P.steps.size(); ++i) {
     const auto own_deps = [&] {
@@ -249,7 +252,8 @@ struct vl_batch {
   int64_t bytes = 0;
   std::vector<vl_image*> images;        // waited on before every run
   DevBlockPtr trace;                    // optional step timeline
-  std::vector<int32_t> trace_meta;      // {job, step, kind} per timeline entry
+  struct TraceStep { int32_t job, step, kind, first, count; };
+  std::vector<TraceStep> trace_steps;   // a plan's step and its steps of the launch
   // A lone job with a tiny plan runs in the per-operator form captured in
   // the graph instead (the persistent launch's step latencies would
   // dominate it): its plan, images and shape.
@@ -636,12 +640,12 @@ vl_status batch_build(vl_context* ctx, const vl_job* jobs, int n_jobs, cudaStrea
     e = dev_alloc(ctx, sizeof(unsigned long long) * 4 * std::max(1, total_steps), st, &b->trace);
     if (e) return cuda_err(ctx, e, "allocating the step timeline");
     L.trace = static_cast<unsigned long long*>(b->trace->ptr);
-    for (int j = 0; j < n_jobs; ++j)
-      for (size_t s2 = 0; s2 < F[J[j].formula_idx].steps.size(); ++s2) {
-        b->trace_meta.push_back(j);
-        b->trace_meta.push_back((int32_t)s2);
-        b->trace_meta.push_back(F[J[j].formula_idx].steps[s2].kind);
-      }
+    for (int j = 0; j < n_jobs; ++j) {
+      const DevSteps& D = F[J[j].formula_idx];
+      for (size_t q = 0, first = 0; q < D.at.size(); first = D.at[q++] + 1)
+        b->trace_steps.push_back({j, (int32_t)q, D.steps[D.at[q]].kind, J[j].step_base + (int32_t)first,
+                                  D.at[q] + 1 - (int32_t)first});
+    }
   }
   // ---- results
   b->done = std::make_shared<EventHolder>();
@@ -1653,18 +1657,28 @@ VL_API vl_status vl_batch_trace(const vl_batch* b, int64_t* out, int64_t max_ent
   if (!valid(b, TAG_BAT)) return VL_ERR_ARG;
   if (!b->trace) return set_err(b->ctx, VL_ERR_ARG, "the batch's context was made without trace");
   DeviceGuard dg(b->ctx->device);
-  const int64_t n = (int64_t)b->trace_meta.size() / 3;
+  const int64_t n = (int64_t)b->trace_steps.size();
   if (n_entries) *n_entries = n;
   if (!out) return VL_OK;
-  std::vector<unsigned long long> t(4 * (size_t)n);
+  std::vector<unsigned long long> t(b->trace->bytes / 8);
   cudaError_t e = cudaEventSynchronize(b->done->ev);
   if (!e) e = cudaMemcpy(t.data(), b->trace->ptr, t.size() * 8, cudaMemcpyDeviceToHost);
   if (e) return cuda_err(b->ctx, e, "reading the step timeline");
   for (int64_t i = 0; i < std::min(n, max_entries); ++i) {
-    out[7 * i + 0] = b->trace_meta[3 * i + 0];
-    out[7 * i + 1] = b->trace_meta[3 * i + 1];
-    out[7 * i + 2] = b->trace_meta[3 * i + 2];
-    for (int k = 0; k < 4; ++k) out[7 * i + 3 + k] = (int64_t)t[4 * i + k];
+    const vl_batch::TraceStep& q = b->trace_steps[i];
+    const unsigned long long* a = &t[4 * (size_t)q.first];
+    unsigned long long v[4] = {a[0], a[1], a[2], a[3]};
+    for (int k = 1; k < q.count; ++k) {  // (a percentile step's passes)
+      a += 4;
+      v[0] = std::min(v[0], a[0]);
+      v[1] = std::max(v[1], a[1]);
+      v[2] += a[2];
+      v[3] += a[3];
+    }
+    out[7 * i + 0] = q.job;
+    out[7 * i + 1] = q.step;
+    out[7 * i + 2] = q.kind;
+    for (int k = 0; k < 4; ++k) out[7 * i + 3 + k] = (int64_t)v[k];
   }
   return VL_OK;
 }
