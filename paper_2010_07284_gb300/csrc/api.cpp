@@ -92,6 +92,23 @@ cudaError_t record_ready(vl_image* im, cudaStream_t st) {
   return e;
 }
 
+static inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
+
+JobBuffers job_buffers(const Plan& P, int H, int W, int cth) {
+  JobBuffers b{};
+  const int Wp = words_per_row(W);
+  const size_t mask = (size_t)H * Wp * 4;
+  const size_t tiles = (size_t)ccl_tiles_y(H, 0, cth) * ccl_tiles_x(Wp);
+  b.pct = align_up(sizeof(float) * std::max(1, P.n_pct_slots), 256);
+  b.planes = align_up(mask * P.n_planes, 256);
+  b.num = align_up(sizeof(float) * (size_t)H * 32 * Wp * P.n_num_images, 256);
+  b.slots = align_up(mask * P.n_inter_slots, 256);
+  b.set_state = align_up(2 * (size_t)H * W * 4, 256);
+  b.set_bytes = b.set_state + align_up(tiles * ccl_tile_cap_host(Wp, cth) * 4, 256);
+  b.sets = b.set_bytes * (size_t)P.n_scratch_sets;
+  return b;
+}
+
 }  // namespace vl
 
 namespace {
@@ -110,7 +127,6 @@ struct DeviceGuard {
 };
 
 inline cudaStream_t S(void* s) { return reinterpret_cast<cudaStream_t>(s); }
-inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 bool valid(const void* h, uint32_t tag) {
   return h && *reinterpret_cast<const uint32_t*>(h) == tag;
@@ -279,7 +295,8 @@ vl_status batch_build(vl_context* ctx, const vl_job* jobs, int n_jobs, cudaStrea
     int H, W, Wp, pitch;
     int gty, gtx, cty, ctx_, ctiles, cth, sel_blocks;
     std::vector<int> need;
-    size_t off_images, off_slotptrs, off_pct, off_slots, off_rz, set_bytes, set_off[2];
+    JobBuffers buf;
+    size_t off_images, off_slotptrs, off_pct, off_slots, off_rz;
     size_t off_roots, off_status, off_planes, off_num, off_hist;
     int n_table;  // image table: the formula's images, then its number images
     int step_base;
@@ -329,7 +346,7 @@ vl_status batch_build(vl_context* ctx, const vl_job* jobs, int n_jobs, cudaStrea
     n_selects += (int64_t)J[j].P->pct.size();
     if (!J[j].P->pct.empty()) select_px = std::max<int64_t>(select_px, (int64_t)J[j].H * J[j].W);
   }
-  const bool split_selects = n_selects > 0 && n_selects < grid && select_px >= (1 << 18);
+  const bool split_selects = n_selects > 0 && n_selects < grid && select_px >= SEL_SPLIT_PIXELS;
   std::vector<DevSteps> F;
   for (const Plan* P : formulas) F.push_back(device_steps(*P, split_selects));
   std::vector<size_t> f_insns(formulas.size()), f_rz(formulas.size()),
@@ -409,7 +426,6 @@ vl_status batch_build(vl_context* ctx, const vl_job* jobs, int n_jobs, cudaStrea
     std::vector<WorkItem> pending;  // every item, step by step
     std::vector<SchedJob> sj(n_jobs);
     for (int j = 0; j < n_jobs; ++j) {
-      const Plan& P = *J[j].P;
       const DevSteps& D = F[J[j].formula_idx];
       sj[j].dep_off = D.dep_off.data();
       sj[j].deps = D.deps.data();
@@ -475,23 +491,12 @@ vl_status batch_build(vl_context* ctx, const vl_job* jobs, int n_jobs, cudaStrea
   // buffers
   for (int j = 0; j < n_jobs; ++j) {
     JobInfo& I = J[j];
-    const Plan& P = *I.P;
-    const size_t mask_bytes = (size_t)I.H * I.Wp * 4;
-    const size_t P_px = (size_t)I.H * I.W;
-    I.off_pct = take(sizeof(float) * std::max(1, P.n_pct_slots));
-    I.off_planes = take(mask_bytes * P.n_planes);
-    I.off_num = take(sizeof(float) * (size_t)I.H * I.pitch * P.n_num_images);
-    I.off_slots = take(mask_bytes * P.n_inter_slots);
-    const size_t tstate = (size_t)I.ctiles * ccl_tile_cap_host(I.Wp, I.cth);
-    // select scratch sets: G (2 * P_px keys) and the tiles' state, 256-byte aligned
-    {
-      size_t o = 0;
-      auto sub = [&](size_t bytes) { o = align_up(o, 256); size_t r = o; o += bytes; return r; };
-      I.set_off[0] = sub(2 * P_px * 4);
-      I.set_off[1] = sub(tstate * 4);
-      I.set_bytes = align_up(o, 256);
-      I.off_rz = take(I.set_bytes * (size_t)P.n_scratch_sets);
-    }
+    I.buf = job_buffers(*I.P, I.H, I.W, I.cth);
+    I.off_pct = take(I.buf.pct);
+    I.off_planes = take(I.buf.planes);
+    I.off_num = take(I.buf.num);
+    I.off_slots = take(I.buf.slots);
+    I.off_rz = take(I.buf.sets);
   }
   const size_t trans_bytes = align_up(off, 256);
   // persistent block: root buffers and status words
@@ -591,8 +596,8 @@ vl_status batch_build(vl_context* ctx, const vl_job* jobs, int n_jobs, cudaStrea
     d.n_rtab = (int32_t)P.rtab.size();
     d.planes = reinterpret_cast<uint32_t*>(tb + I.off_planes);
     d.rzs = reinterpret_cast<unsigned char*>(tb + I.off_rz);
-    d.set_bytes = (int64_t)I.set_bytes;
-    d.off_state = (int64_t)I.set_off[1];
+    d.set_bytes = (int64_t)I.buf.set_bytes;
+    d.off_state = (int64_t)I.buf.set_state;
     d.tile_cap = ccl_tile_cap_host(I.Wp, I.cth);
     d.c_th = I.cth;
     d.status = status_dev + j;

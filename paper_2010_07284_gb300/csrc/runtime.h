@@ -115,6 +115,15 @@ struct vl_batch;
 
 namespace vl {
 
+// Device memory of one job of a batch besides its tables and result masks:
+// the parts as batch_build lays them out, 256-byte aligned each.
+struct JobBuffers {
+  size_t pct, planes, num, slots;
+  size_t set_state, set_bytes;  // a select scratch set: union-find, then the tiles' state
+  size_t sets;                  // all of them
+};
+JobBuffers job_buffers(const Plan& P, int H, int W, int cth);
+
 // Helpers shared by api.cpp and server.cpp.
 vl_status set_err(vl_context* ctx, vl_status code, const std::string& msg);
 vl_status cuda_err(vl_context* ctx, cudaError_t e, const char* what);

@@ -46,17 +46,14 @@ struct Flight {
 
 inline size_t align256(size_t x) { return (x + 255) / 256 * 256; }
 
-// Device bytes one query needs inside a batch (mirrors the batch layout:
-// slots, percentile values, select scratch, result masks, tables).
+// Device bytes one query needs inside a batch: its buffers as the batch lays
+// them out, the state of its percentile selects if many blocks share them,
+// result masks, and its tables by their largest parts.
 int64_t estimate_bytes(const Plan& P, int H, int W) {
-  const int Wp = words_per_row(W);
-  const size_t mask = (size_t)H * Wp * 4, px = (size_t)H * W;
-  const size_t tiles = (size_t)ccl_tiles_y(H) * ccl_tiles_x(Wp);
-  const size_t tstate = tiles * ccl_tile_cap_host(Wp);
-  size_t b = align256(mask * (P.n_inter_slots + P.n_root_slots));
-  b += (size_t)P.n_scratch_sets *
-       (align256(2 * px * 4) + align256(tstate * 4) + align256(tstate));
-  b += align256(sizeof(uint32_t) * SEL_HIST * P.pct.size());
+  const JobBuffers B = job_buffers(P, H, W, CCL_TH);
+  size_t b = B.pct + B.planes + B.num + B.slots + B.sets;
+  b += align256((size_t)H * words_per_row(W) * 4 * P.n_root_slots);
+  if ((int64_t)H * W >= SEL_SPLIT_PIXELS) b += align256(sizeof(uint32_t) * SEL_HIST * P.pct.size());
   b += align256(sizeof(Insn) * P.insns.size()) + align256(sizeof(StepRec) * (P.steps.size() + SEL_PASSES)) +
        64 * 1024;
   return (int64_t)b;

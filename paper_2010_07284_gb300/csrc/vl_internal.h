@@ -145,6 +145,8 @@ constexpr int RANK_ROWS = 8;
 constexpr int SEL_PASSES = 4;
 constexpr int SEL_BINS = 4096;
 constexpr int SEL_HIST = 16 + SEL_PASSES * SEL_BINS;
+// Channels from which many blocks share a select (batch_build says why).
+constexpr int64_t SEL_SPLIT_PIXELS = 1 << 18;
 static inline int select_blocks(int64_t pixels, int64_t side_by_side, int64_t slots) {
   int64_t n = slots / side_by_side, most = (pixels + 8191) / 8192;
   if (n > most) n = most;
