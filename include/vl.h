@@ -95,10 +95,10 @@ typedef struct {
                              a reserve */
   int32_t tile_rows;      /* 0 = autotune; else rows per fused tile (<= 1024) */
   int32_t tile_words;     /* 0 = autotune; else 32-px words per fused tile
-                             (<= 256).  VL_ERR_ARG when four buffers of
-                             tile_rows + 16 rows of tile_words words, rounded up
-                             to whole fours, and eight more do not fit one
-                             CTA's shared memory (227 KB on sm_103a) */
+                             (<= 256).  VL_ERR_ARG when (tile_rows + 16) *
+                             (tile_words + 2) is above 6720.  Tiles run with
+                             their words rounded up to a multiple of four, and
+                             tall ones in equal parts */
   int32_t reserved[6];
 } vl_config;
 

@@ -327,15 +327,15 @@ vl_status batch_build(vl_context* ctx, const vl_job* jobs, int n_jobs, cudaStrea
   size_t off = 0;
   auto take = [&](size_t bytes, size_t a = 256) { off = align_up(off, a); size_t o = off; off += bytes; return o; };
   const size_t off_jobs = take(sizeof(DevJob) * n_jobs);
-  const TileShape ts = force ? *force : pick_tile_shape(ctx, jobs, n_jobs, nullptr, !persistent);
+  TileShape ts = force ? *force : pick_tile_shape(ctx, jobs, n_jobs, nullptr, !persistent);
   if (ts.per_op) {
     if (n_jobs != 1 || persistent)
       return set_err(ctx, VL_ERR_ARG, "the per-operator form takes a batch of one job");
     return batch_build_per_op(ctx, jobs[0], J[0].H, J[0].W, st, out);
   }
   if (!tile_shape_fits(ctx, ts)) return set_err(ctx, VL_ERR_ARG, "tile shape does not fit shared memory");
-  const int fit = tile_shape_ctas(ctx, ts);
-  const int cps = ts.ctas_per_sm > 0 ? std::min(ts.ctas_per_sm, fit) : fit;
+  ts = tile_run_shape(ctx, ts);
+  const int cps = ts.ctas_per_sm > 0 ? std::min(ts.ctas_per_sm, ctx->ctas_per_sm) : ctx->ctas_per_sm;
   const int grid = std::max(1, ctx->sm_count * cps);
   // A percentile select is one block's work when there are as many as blocks,
   // or the channels are small: five selects of one 256 x 256 image take 30 us
@@ -639,7 +639,7 @@ vl_status batch_build(vl_context* ctx, const vl_job* jobs, int n_jobs, cudaStrea
   L.spin_limit = ctx->cfg.spin_limit != 0 ? ctx->cfg.spin_limit : (1LL << 22);
   L.group_buffers = ctx->nb;
   L.grid = std::max(1, std::min<int>(grid, (int)items.size()));
-  L.smem_bytes = (int32_t)tile_shape_smem(ctx, ts);
+  L.smem_bytes = (int32_t)ctx->exec_smem;
   L.trace = nullptr;
   if (ctx->cfg.trace) {
     e = dev_alloc(ctx, sizeof(unsigned long long) * 4 * std::max(1, total_steps), st, &b->trace);
@@ -1147,16 +1147,21 @@ VL_API vl_status vl_context_create(const vl_config* cfg, vl_context** out) {
     delete c;
     return VL_ERR_ARG;
   }
-  c->gth = c->cfg.tile_rows > 0 ? c->cfg.tile_rows : 32;
-  c->gtww = c->cfg.tile_words > 0 ? c->cfg.tile_words : 32;
   c->hmax = 8;
+  TileShape fixed{};
+  if (c->cfg.tile_rows > 0) {
+    // (which shapes are refused is a measure of its own: four buffers with one
+    // word either side in the budget)
+    fixed.rows = c->cfg.tile_rows;
+    fixed.words = c->cfg.tile_words;
+    if (16LL * (fixed.rows + 2 * c->hmax) * (fixed.words + 2) > kGroupBudget) { delete c; return VL_ERR_ARG; }
+    fixed = tile_run_shape(fixed, c->hmax, EXEC_THREADS);
+  }
+  c->gth = fixed.rows;
+  c->gtww = fixed.words;
   const int bh = c->gth + 2 * c->hmax;
-  if ((e = exec_max_smem(c->device, &c->exec_smem_max))) { delete c; cudaGetLastError(); return VL_ERR_CUDA; }
   c->nb = (int)std::min<int64_t>(64, kGroupBudget / group_buffer_bytes(bh, c->gtww));
-  // (a plan needs four buffers: tiles too tall for that many in the budget may
-  // take a whole SM's shared memory)
-  c->nb = std::max(c->nb, 4);
-  if (exec_smem_bytes(c->nb, bh, c->gtww) > c->exec_smem_max) { delete c; return VL_ERR_ARG; }
+  if (c->nb < 4) { delete c; return VL_ERR_ARG; }
   c->pp.group_buffers = c->nb;
   c->pp.hmax = c->hmax;
   c->exec_smem = exec_smem_bytes(c->nb, bh, c->gtww);
@@ -1174,11 +1179,11 @@ VL_API vl_status vl_context_create(const vl_config* cfg, vl_context** out) {
       if (two > c->exec_smem && two <= (size_t)optin) c->exec_smem = two;
     }
   }
-  if ((e = exec_occupancy(c->exec_smem, &c->ctas_per_sm))) { delete c; cudaGetLastError(); return VL_ERR_CUDA; }
+  if ((e = exec_configure(c->exec_smem, &c->ctas_per_sm))) { delete c; cudaGetLastError(); return VL_ERR_CUDA; }
   if (c->ctas_per_sm < 2 && c->exec_smem > exec_smem_bytes(c->nb, bh, c->gtww)) {
     // the widened size lost the second CTA on this GPU: fall back
     c->exec_smem = exec_smem_bytes(c->nb, bh, c->gtww);
-    if ((e = exec_occupancy(c->exec_smem, &c->ctas_per_sm))) { delete c; cudaGetLastError(); return VL_ERR_CUDA; }
+    if ((e = exec_configure(c->exec_smem, &c->ctas_per_sm))) { delete c; cudaGetLastError(); return VL_ERR_CUDA; }
   }
   if (c->ctas_per_sm < 1) c->ctas_per_sm = 1;
   if ((e = cudaMalloc(&c->ccl_status, sizeof(int32_t)))) { delete c; cudaGetLastError(); return VL_ERR_OOM; }

@@ -15,7 +15,6 @@
 #include <iterator>
 #include <set>
 
-#include "kernels.h"
 #include "runtime.h"
 
 namespace vl {
@@ -81,8 +80,7 @@ vl_tile_choice to_choice(const vl_context* ctx, const TileShape& t, int status, 
   c.tile_rows = t.per_op ? 0 : t.rows;
   c.tile_words = t.per_op ? 0 : t.words;
   c.ctas_per_sm = t.per_op ? 0
-                  : t.ctas_per_sm > 0 ? std::min(t.ctas_per_sm, tile_shape_ctas(ctx, t))
-                                      : tile_shape_ctas(ctx, t);
+                  : t.ctas_per_sm > 0 ? std::min(t.ctas_per_sm, ctx->ctas_per_sm) : ctx->ctas_per_sm;
   c.status = status;
   c.ms = ms;
   return c;
@@ -100,22 +98,41 @@ uint64_t plan_hash(const Plan& P) {
   return h;
 }
 
-size_t tile_shape_smem(const vl_context* ctx, const TileShape& t) {
-  return std::max(ctx->exec_smem, exec_smem_bytes(ctx->nb, t.rows + 2 * ctx->hmax, t.words));
+// Words are rounded up to whole vectors: the buffers have room for those anyway,
+// and masks have rows of them, so that tiles start on 16-byte boundaries.  A
+// tile with more rows than give each thread of the block one vector (with the
+// halo rows) is cut into equal parts that do, unless these would have fewer
+// rows than their halo on one side: the interpreter's fast path is for one
+// vector a thread.  (1000 nodes at 2048 x 2048, with the shapes as asked for
+// and as they run: 33 x 7 words FIG33A and FIG33B ms, 256 x 4 FIG256A and FIG256B, 64 x 32
+// FIG64A and FIG64B.)
+TileShape tile_run_shape(const TileShape& t, int hmax, int64_t max_vecs) {
+  TileShape r = t;
+  r.words = (t.words + 3) & ~3;
+  const int most = (int)(std::min<int64_t>(max_vecs, EXEC_THREADS) / group_vecs(r.words)) - 2 * hmax;
+  if (r.rows > most && most >= hmax) {
+    const int parts = (r.rows + most - 1) / most;
+    r.rows = (r.rows + parts - 1) / parts;
+  }
+  return r;
 }
+TileShape tile_run_shape(const vl_context* ctx, const TileShape& t) {
+  return tile_run_shape(t, ctx->hmax, ((int64_t)ctx->exec_smem - GROUP_PROG_BYTES) / (16 * ctx->nb));
+}
+
 bool tile_shape_fits(const vl_context* ctx, const TileShape& t) {
-  return t.rows >= 1 && t.words >= 1 && tile_shape_smem(ctx, t) <= ctx->exec_smem_max;
-}
-// (exec_smem is what two CTAs of an SM can have, or more)
-int tile_shape_ctas(const vl_context* ctx, const TileShape& t) {
-  return tile_shape_smem(ctx, t) > ctx->exec_smem ? 1 : ctx->ctas_per_sm;
+  if (t.rows < 1 || t.words < 1) return false;
+  const TileShape r = tile_run_shape(ctx, t);
+  const int64_t bytes =
+      GROUP_PROG_BYTES + ctx->nb * group_buffer_bytes(r.rows + 2 * ctx->hmax, r.words);
+  return bytes <= (int64_t)ctx->exec_smem;
 }
 
 // Shapes that a tile table may name and the autotuner tries: the tile's words
 // with one beside them on either side, for every buffer of a plan, in half an
 // SM's shared memory.  A measure of its own, so that which tables load does
 // not depend on how the buffers are laid out; a shape whose buffers then do
-// not fit (a tall tile of a few words) is passed over when a batch is built.
+// not fit (a low tile of many words) is passed over when a batch is built.
 constexpr int64_t kTableSmem = 115456;
 static bool tile_shape_in_table(const vl_context* ctx, const TileShape& t) {
   return t.rows >= 1 && t.words >= 1 &&
@@ -216,7 +233,6 @@ extern "C" VL_API vl_status vl_autotune(vl_context* ctx, const vl_job* jobs, int
   for (const TileShape& base : bases) {
     if (!tile_shape_in_table(ctx, base) || !tile_shape_fits(ctx, base)) continue;
     for (int cps : cps_list) {
-      if (cps > tile_shape_ctas(ctx, base)) continue;
       TileShape t = base;
       t.ctas_per_sm = cps;
       cands.push_back(t);

@@ -31,8 +31,9 @@ VL_DEV void group_sync(int n) { asm volatile("bar.sync 1, %0;" ::"r"(n) : "memor
 
 // One tile of a group, as its threads see it.
 //
-// Buffers are rows of nv vectors of four words: the core tile's words, and a
-// whole vector left and right of them (only the word next to the core
+// Buffers are rows of nv vectors of four words: the core tile's words (tiles
+// have whole vectors of them), and a
+// vector left and right of them (only the word next to the core
 // matters: a halo is at most 31 pixels), so that every vector of a buffer
 // starts at a 16-byte boundary of the mask it comes from.  Vector v of every
 // buffer belongs to thread v mod EXEC_THREADS, for every instruction except
@@ -57,29 +58,26 @@ VL_DEV GroupGeom group_geom(const DevJob& J, const StepDesc& S, int sub) {
   return g;
 }
 
-// Vector v of the buffers.  ALIGNED: tile words come in fours, so a vector
-// lies in the image's words whole or not at all.
+// Vector v of the buffers: it lies in the image's words whole or not at all.
 struct GroupVec {
   int at;        // first word in a buffer
   int off;       // first word in a mask of the image
   int need;      // halo from which it is computed; huge: no such vector
   int row;       // the same for its row as a whole
-  int lo, hi;    // its pixels [lo, hi) lie in the image (none: lo >= hi)
+  int hi;        // its pixels [0, hi) lie in the image (none: hi <= 0)
   int where;     // bit 0: first of its row, bit 1: last
-  int core;      // words of it in the core tile
-  VL_DEV bool in() const { return lo < hi; }
+  bool core;     // its words are the core tile's
+  VL_DEV bool in() const { return hi > 0; }
   // the pixels of word k that lie in the image
   VL_DEV uint32_t mask(int k) const {
     const int n = hi - 32 * k;
-    const uint32_t m = n >= 32 ? 0xFFFFFFFFu : n <= 0 ? 0u : (1u << n) - 1u;
-    return lo > 32 * k ? 0u : m;  // (a word left of the image; words are whole there)
+    return n >= 32 ? 0xFFFFFFFFu : n <= 0 ? 0u : (1u << n) - 1u;
   }
   VL_DEV uint4 clip(uint4 v) const {
-    if (lo == 0 && hi == 128) return v;
+    if (hi == 128) return v;
     return make_uint4(v.x & mask(0), v.y & mask(1), v.z & mask(2), v.w & mask(3));
   }
 };
-template <bool ALIGNED>
 VL_DEV GroupVec group_vec(const DevJob& J, const GroupGeom& g, int v) {
   GroupVec q;
   const int i = v / g.nv, jv = v - i * g.nv;
@@ -90,38 +88,17 @@ VL_DEV GroupVec group_vec(const DevJob& J, const GroupGeom& g, int v) {
   q.row = i < g.rows ? max(g.halo - i, i - (g.halo + g.th - 1)) : 1 << 20;
   q.need = max(q.row, q.where ? 1 : 0);
   const int y = g.r0 - g.halo + i, wg = g.w0 - 4 + 4 * jv;
-  q.hi = y >= 0 && y < J.H ? min(128, J.W - 32 * wg) : 0;
-  q.lo = 0;
-  if (wg < 0) {
-    if (ALIGNED) q.hi = 0;
-    else q.lo = -32 * wg;
-  }
+  q.hi = y >= 0 && y < J.H && wg >= 0 ? min(128, J.W - 32 * wg) : 0;
   q.off = y * J.Wp + wg;
-  q.core = q.need <= 0 ? max(0, min(4, g.tww - 4 * (jv - 1))) : 0;
+  q.core = q.need <= 0 && 4 * (jv - 1) < g.tww;
   return q;
 }
 // Its words of the mask at g (0 outside the image), and back.
-template <bool ALIGNED>
 VL_DEV uint4 vec_load(const uint32_t* g, const GroupVec& q) {
-  uint4 v = make_uint4(0u, 0u, 0u, 0u);
-  if (!q.in()) return v;
-  if (ALIGNED) return __ldcg(reinterpret_cast<const uint4*>(g + q.off));
-  if (q.mask(0)) v.x = ldcg(g + q.off);
-  if (q.mask(1)) v.y = ldcg(g + q.off + 1);
-  if (q.mask(2)) v.z = ldcg(g + q.off + 2);
-  if (q.mask(3)) v.w = ldcg(g + q.off + 3);
-  return v;
+  return q.in() ? __ldcg(reinterpret_cast<const uint4*>(g + q.off)) : make_uint4(0u, 0u, 0u, 0u);
 }
-template <bool ALIGNED>
 VL_DEV void vec_store(uint32_t* g, const GroupVec& q, uint4 v) {
-  if (ALIGNED) {
-    if (q.core) *reinterpret_cast<uint4*>(g + q.off) = v;
-    return;
-  }
-  if (q.core > 0) g[q.off] = v.x;
-  if (q.core > 1) g[q.off + 1] = v.y;
-  if (q.core > 2) g[q.off + 2] = v.z;
-  if (q.core > 3) g[q.off + 3] = v.w;
+  if (q.core) *reinterpret_cast<uint4*>(g + q.off) = v;
 }
 
 // Instructions as the interpreter runs them, four words each:
@@ -215,7 +192,6 @@ VL_DEV int stage_at(const StepDesc& S, const GroupGeom& g, const GroupVec& q) {
   const int v = q.at >> 2, i = v / g.nv, jv = v - i * g.nv;
   return ((i - (g.halo - S.rank_halo)) * (g.nv - 1) + (q.where ? g.nv - 2 : jv - 1)) * 4;
 }
-template <bool ALIGNED>
 VL_DEV void stage_copy(const DevJob& J, const StepDesc& S, const GroupGeom& g, const GroupVec& q,
                        uint32_t* stage) {
   if (q.need > S.rank_halo || !q.in()) return;
@@ -230,11 +206,8 @@ VL_DEV void stage_copy(const DevJob& J, const StepDesc& S, const GroupGeom& g, c
         if (q.mask(3)) cp_async4(dst + 3, src + 3);
       } else if (q.where) {
         if (q.mask(0)) cp_async4(dst, src);
-      } else if (ALIGNED) {
-        cp_async16(dst, src);
       } else {
-        for (int k = 0; k < 4; ++k)
-          if (q.mask(k)) cp_async4(dst + k, src + k);
+        cp_async16(dst, src);
       }
     }
   }
@@ -258,7 +231,6 @@ VL_DEV uint4 rank_result(uint4 w, uint4 nan, bool lt) {
 
 // The value of instruction I (no load, store or float threshold) on vector q.
 // stage: the thread's place in the staged planes.
-template <bool ALIGNED>
 VL_DEV uint4 group_value(const DevJob& J, uint4 I, uint32_t op, const uint32_t* buf,
                          const GroupVec& q, int row_words, const uint32_t* stage, int per_plane) {
   const uint32_t* const a = buf + (I.x >> 16) * 4 + q.at;
@@ -302,8 +274,8 @@ VL_DEV uint4 group_value(const DevJob& J, uint4 I, uint32_t op, const uint32_t* 
       const uint32_t* g = J.planes + (size_t)I.w * pstride;
 #pragma unroll 4
       for (int b = b0; b < nb; ++b)
-        rank_pass(w, vec_load<ALIGNED>(g + (size_t)b * pstride, q), 0u - ((K >> b) & 1u));
-      if (lt) nan = vec_load<ALIGNED>(g + (size_t)nb * pstride, q);
+        rank_pass(w, vec_load(g + (size_t)b * pstride, q), 0u - ((K >> b) & 1u));
+      if (lt) nan = vec_load(g + (size_t)nb * pstride, q);
     }
     z = rank_result(w, nan, lt);
   }
@@ -417,7 +389,7 @@ VL_DEV const uint32_t* group_run(const DevJob& J, const uint32_t* prog, const ui
     pc += 4;
     next = lds4(pc);
     if (op == P_STORE) {
-      if (own.core) vec_store<true>(insn_ptr(I), own, lds4(buf + (I.x >> 16) * 4 + own.at));
+      if (own.core) vec_store(insn_ptr(I), own, lds4(buf + (I.x >> 16) * 4 + own.at));
       continue;
     }
     const bool mine = own.need <= (int)((I.y >> 16) & 0x7Fu);
@@ -427,7 +399,7 @@ VL_DEV const uint32_t* group_run(const DevJob& J, const uint32_t* prog, const ui
         cp_async_wait<DEPTH ? DEPTH - 1 : 0>();  // the oldest fetch has landed
         if (mine && own.in()) z = lds4(ring.base + (load & (DEPTH - 1)) * ring.entry);
       } else if (mine) {
-        z = vec_load<true>(insn_ptr(I), own);
+        z = vec_load(insn_ptr(I), own);
       }
     } else if (op == P_NEAR) {
       // the words beside the vector come from the lanes that hold the vectors
@@ -454,11 +426,11 @@ VL_DEV const uint32_t* group_run(const DevJob& J, const uint32_t* prog, const ui
       z = own.clip(near_vec(x, o, l, e));
     } else if (mine) {
       if (op == P_RTHR) cp_async_wait<DEPTH>();  // the staged planes have landed
-      z = group_value<true>(J, I, op, buf, own, row_words, stage, per_plane);
+      z = group_value(J, I, op, buf, own, row_words, stage, per_plane);
     }
     if (mine) sts4(buf + (I.x & 0xFFFFu) * 4 + own.at, z);
     if (I.y & P_PUT) {
-      if (own.core) vec_store<true>(insn_ptr(next), own, z);
+      if (own.core) vec_store(insn_ptr(next), own, z);
       pc += 4;
       next = lds4(pc);
     }
@@ -466,9 +438,8 @@ VL_DEV const uint32_t* group_run(const DevJob& J, const uint32_t* prog, const ui
   }
 }
 
-// The same for any tile: also one with more vectors than threads, or whose
-// words are no multiple of four (its vectors then cross 16-byte boundaries,
-// and masks are read and written word by word).
+// The same for a tile with more vectors than threads (one of many words, see
+// tile_run_shape).
 static __device__ __noinline__ void group_run_any(const DevJob& J, const StepDesc& S, int sub,
                                                   const uint32_t* prog, uint32_t* buf,
                                                   const uint32_t* stage) {
@@ -486,12 +457,12 @@ static __device__ __noinline__ void group_run_any(const DevJob& J, const StepDes
       continue;
     }
     for (int v = threadIdx.x; v < n; v += EXEC_THREADS) {
-      const GroupVec q = group_vec<false>(J, g, v);
+      const GroupVec q = group_vec(J, g, v);
       if (op == P_STORE) {
-        vec_store<false>(insn_ptr(I), q, lds4(buf + (I.x >> 16) * 4 + q.at));
+        vec_store(insn_ptr(I), q, lds4(buf + (I.x >> 16) * 4 + q.at));
       } else if (q.need <= (int)((I.y >> 16) & 0x7Fu)) {
-        sts4(d + q.at, op == P_LOAD ? vec_load<false>(insn_ptr(I), q)
-                                    : group_value<false>(J, I, op, buf, q, g.nv * 4,
+        sts4(d + q.at, op == P_LOAD ? vec_load(insn_ptr(I), q)
+                                    : group_value(J, I, op, buf, q, g.nv * 4,
                                                          stage + stage_at(S, g, q), per_plane));
       }
     }
@@ -505,7 +476,7 @@ VL_DEV void group_tile(const DevJob& J, const StepDesc& S, int sub, uint32_t* sm
   constexpr int DEPTH = 4;
   const int tid = threadIdx.x, lane = tid & 31, n_insn = S.insn_cnt;
   const GroupGeom g = group_geom(J, S, sub);
-  const bool one = (J.gtww & 3) == 0 && g.rows * g.nv <= EXEC_THREADS;
+  const bool one = g.rows * g.nv <= EXEC_THREADS;
   // threads that take part (a float threshold takes all); the others leave
   const int n_act = one && S.pct_cnt == 0 ? (g.rows * g.nv + 31) & ~31 : EXEC_THREADS;
   if (tid >= n_act) return;
@@ -513,18 +484,18 @@ VL_DEV void group_tile(const DevJob& J, const StepDesc& S, int sub, uint32_t* sm
   uint32_t* const buf = smem + GROUP_PROG_BYTES / 4;
   uint32_t* rest = buf + min(max(S.n_bufs, 1), buffers) * g.vecs * 4;
   int room = smem_words - (int)(rest - smem);
-  const GroupVec own = group_vec<true>(J, g, tid);
+  const GroupVec own = group_vec(J, g, tid);
   // the planes of the group's rank tables, when they fit
   const int st_words = stage_words(J, S, g, 32);
   const bool staged = S.rank_mask && st_words <= room;
   const uint32_t* stage = rest;
   if (staged) {
     if (one) {
-      stage_copy<true>(J, S, g, own, rest);
+      stage_copy(J, S, g, own, rest);
       stage += stage_at(S, g, own);
     } else {
       for (int v = tid; v < g.rows * g.nv; v += EXEC_THREADS)
-        stage_copy<false>(J, S, g, group_vec<false>(J, g, v), rest);
+        stage_copy(J, S, g, group_vec(J, g, v), rest);
     }
     rest += st_words;
     room -= st_words;

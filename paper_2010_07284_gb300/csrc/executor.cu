@@ -410,17 +410,10 @@ size_t exec_smem_bytes(int group_buffers, int group_rows, int tile_words) {
   return (m + 15) & ~(size_t)15;
 }
 
-cudaError_t exec_max_smem(int device, size_t* bytes) {
-  int optin = 0;
-  cudaFuncAttributes a{};
-  cudaError_t e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
-  if (!e) e = cudaFuncGetAttributes(&a, k_exec);
+cudaError_t exec_configure(size_t smem_bytes, int* max_ctas_per_sm) {
+  cudaError_t e = cudaFuncSetAttribute(k_exec, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)smem_bytes);
   if (e) return e;
-  *bytes = ((size_t)optin - a.sharedSizeBytes) & ~(size_t)127;
-  return cudaFuncSetAttribute(k_exec, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)*bytes);
-}
-
-cudaError_t exec_occupancy(size_t smem_bytes, int* max_ctas_per_sm) {
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(max_ctas_per_sm, k_exec, EXEC_THREADS,
                                                        smem_bytes);
 }

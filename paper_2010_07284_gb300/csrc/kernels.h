@@ -142,11 +142,7 @@ struct ExecLaunch {
 };
 // group_rows: rows of a buffer (tile rows + 2 * the largest halo).
 size_t exec_smem_bytes(int group_buffers, int group_rows, int tile_words);
-// The most dynamic shared memory a CTA of the executor may have; the kernel is
-// set up for it (the setting is one for all contexts of a device).
-cudaError_t exec_max_smem(int device, size_t* bytes);
-// CTAs of the executor an SM holds with that much each.
-cudaError_t exec_occupancy(size_t smem_bytes, int* max_ctas_per_sm);
+cudaError_t exec_configure(size_t smem_bytes, int* max_ctas_per_sm);
 cudaError_t launch_exec(const ExecLaunch& L, cudaStream_t st);
 
 }  // namespace vl

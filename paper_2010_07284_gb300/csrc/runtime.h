@@ -54,8 +54,7 @@ struct vl_context {
   int device = 0;
   int sm_count = 0;
   int ctas_per_sm = 1;
-  size_t exec_smem = 0;      // dynamic shared memory of a CTA, for ctas_per_sm of them
-  size_t exec_smem_max = 0;  // the most one CTA may have
+  size_t exec_smem = 0;
   int gth = 32, gtww = 32, hmax = 8, nb = 14;
   vl::PlanParams pp{};
   int32_t* ccl_status = nullptr;  // device word of vl_ccl
@@ -151,11 +150,12 @@ vl_status plain_enqueue(vl_context* ctx, const Plan& P, vl_image* const* imgs, i
 // allow_per_op = false: only shapes of the persistent executor.
 TileShape pick_tile_shape(vl_context* ctx, const vl_job* jobs, int n_jobs, int* tuned = nullptr,
                           bool allow_per_op = true);
-// Dynamic shared memory a batch with this tile shape is launched with, whether
-// a CTA may have that much, and how many such CTAs an SM holds.
-size_t tile_shape_smem(const vl_context* ctx, const TileShape& t);
+// The tiles a batch runs for a shape that was asked for: words in whole vectors
+// of four, tall tiles in parts.  max_vecs: vectors a buffer may have.
+TileShape tile_run_shape(const TileShape& t, int hmax, int64_t max_vecs);
+TileShape tile_run_shape(const vl_context* ctx, const TileShape& t);
+// Whether the group buffers of those fit the executor's shared memory.
 bool tile_shape_fits(const vl_context* ctx, const TileShape& t);
-int tile_shape_ctas(const vl_context* ctx, const TileShape& t);
 uint64_t plan_hash(const Plan& P);
 vl_status batch_run(vl_batch* b, cudaStream_t st);
 // Hand the batch's results to the caller (they keep the batch memory alive).

@@ -1,7 +1,7 @@
-"""Tile shapes at the edges of what is accepted: tall tiles of few words, whose
-buffers take more shared memory than two CTAs of an SM can have, run and give the
-oracle's masks, beside contexts of other shapes; a tile table may name shapes
-that need that much, and shapes that no longer fit at all."""
+"""Tile shapes at the edges of what is accepted: tall tiles of few words and tiles
+whose words are no multiple of four run and give the oracle's masks, beside
+contexts of other shapes; a tile table may name such shapes, and shapes whose
+buffers do not fit."""
 import re
 
 import numpy as np
@@ -19,7 +19,8 @@ def _formula():
     return wl.formula_to_records(f), f.roots
 
 
-@pytest.mark.parametrize("rows,words", [(545, 1), (1024, 1), (1024, 4), (600, 4), (825, 5), (512, 8), (80, 44)])
+@pytest.mark.parametrize("rows,words", [(545, 1), (1024, 1), (1024, 4), (600, 4), (825, 5), (512, 8), (80, 44),
+                                        (33, 7), (6, 200), (1, 250)])
 def test_tall_tiles_match_oracle(rows, words):
     torch_cuda()
     rec, roots = _formula()
@@ -27,7 +28,7 @@ def test_tall_tiles_match_oracle(rows, words):
     for h, w in ((1100, 131), (70, 1500)):
         img = wl.uniform_image(h, w, seed=h)
         check_formula(rec, roots, [img], ctx=ctx, modes=("fused",))
-        check_formula(rec, roots, [img], ctx=context(), modes=("fused",))  # (another shared size)
+        check_formula(rec, roots, [img], ctx=context(), modes=("fused",))
 
 
 def test_refused_shapes():
@@ -38,9 +39,9 @@ def test_refused_shapes():
             vg.Context(tile_rows=rows, tile_words=words)
 
 
-@pytest.mark.parametrize("rows,words,runs", [(33, 32, True), (34, 32, True), (44, 32, True), (128, 8, True),
-                                             (322, 4, True), (600, 1, False)])
-def test_tables_name_shapes_beyond_two_ctas(tmp_path, rows, words, runs):
+@pytest.mark.parametrize("rows,words,runs", [(33, 32, True), (44, 32, True), (128, 8, True), (20, 7, True),
+                                             (322, 4, True), (600, 1, True), (2, 112, False)])
+def test_tables_name_tall_narrow_and_wide_shapes(tmp_path, rows, words, runs):
     torch_cuda()
     import paper_2010_07284_gb300 as vg
     rec, roots = _formula()
@@ -91,4 +92,4 @@ def test_autotuner_tries_one_wave_heights_again():
     assert 34 <= rows <= 44
     trials = ctx.autotune(jobs, stream=s, reps=1)["trials"]
     tall = [t for t in trials if (t["tile_rows"], t["tile_words"]) == (rows, 32)]
-    assert tall and all(t["status"] == 0 and t["ctas_per_sm"] == 1 for t in tall)
+    assert len(tall) == 2 and all(t["status"] == 0 for t in tall)
