@@ -340,7 +340,11 @@ vl_status batch_build(vl_context* ctx, const vl_job* jobs, int n_jobs, cudaStrea
   // A percentile select is one block's work when there are as many as blocks,
   // or the channels are small: five selects of one 256 x 256 image take 30 us
   // that way and 40 us as passes that many blocks share (five more steps),
-  // of 384 x 384 56 and 48 us, of 512 x 512 about 105 and 44 us.
+  // of 384 x 384 56 and 48 us, of 512 x 512 about 105 and 44 us.  The largest
+  // channel decides for all, and the passes pay up to a block a select: sixty
+  // 240 x 240 images beside one of 520 x 512, three selects each, take 204 us
+  // that way and 188 as passes, beside one of 1024 x 1024 656 and 510; 300
+  // selects of 520 x 512 channels 352 and 321.
   int64_t n_selects = 0, select_px = 0;
   for (int j = 0; j < n_jobs; ++j) {
     n_selects += (int64_t)J[j].P->pct.size();
@@ -433,7 +437,9 @@ vl_status batch_build(vl_context* ctx, const vl_job* jobs, int n_jobs, cudaStrea
       for (size_t si = 0; si < J[j].need.size(); ++si) {
         const StepDesc& sd = D.steps[si];
         const int n = J[j].need[si];
-        // estimated microseconds per sub-item (one GB300, two CTAs per SM)
+        // estimated microseconds per sub-item (one GB300, two CTAs per SM): what
+        // the order needs is their proportions.  (Groups, labelling, final
+        // pass and rank codes were measured on earlier forms of those kernels.)
         double sub_us;
         switch (sd.kind) {
           case SK_GROUP: sub_us = (5.0 + 1.3 * sd.insn_cnt) * tile_scale; break;

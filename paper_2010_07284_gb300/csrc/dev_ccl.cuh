@@ -15,7 +15,8 @@
 //      is linked under the smaller root by compare-and-swap, so only a node
 //      that is still a root is ever re-pointed and links always point to
 //      smaller gids (no cycles).
-//   4. final: each tile relabels again and resolves its border roots in G.
+//   4. final: each tile takes up what it saved, resolves its border roots in
+//      G, and writes labels or the selected components.
 // Labels are canonical: the minimum linear index of each component.
 #pragma once
 #include <climits>
@@ -31,6 +32,7 @@ constexpr int CCL_PEND = 4096;
 static_assert(CCL_MAXRUNS <= 16384, "runs are packed into 16 bits with two flags");
 
 struct CclSmem {
+  static constexpr bool SEEDS = true;
   uint32_t m[CCL_TH][CCL_TWW];   // rows of the tile
   uint32_t u[CCL_NS][CCL_TWW];   // strip unions (row 2k | row 2k+1)
   uint32_t st[CCL_NS][CCL_TWW];  // strip-run starts
@@ -52,10 +54,10 @@ struct CclSmem {
 // RZ_SEED when it holds a seed pixel and RZ_SEL when it is selected).
 constexpr uint32_t RZ_ROOT = 0x8000u, RZ_SEED = 0x4000u, RZ_SEL = 0x2000u;
 struct RzSmem {
+  static constexpr bool SEEDS = false;
   uint32_t m[CCL_TH][CCL_TWW];
   uint32_t u[CCL_NS][CCL_TWW];
   uint32_t st[CCL_NS][CCL_TWW];
-  uint32_t sd[CCL_NS][CCL_TWW];  // (unused)
   int32_t pre[CCL_NS][CCL_TWW];
   int32_t cnt[CCL_NS];
   int32_t base[CCL_NS + 1];
@@ -304,10 +306,6 @@ VL_DEV int sid(const Smem& s, int k, int x) {
   return s.base[k] + s.pre[k][w] + __popc(s.st[k][w] & le_mask(x & 31)) - 1;
 }
 
-VL_DEV bool mbit(const CclSmem& s, int row, int x) {
-  return (s.m[row][x >> 5] >> (x & 31)) & 1u;
-}
-
 // Root of strip run i once roots are encoded (parent[root] < 0).
 VL_DEV int root_of(const CclSmem& s, int i) {
   const int p = s.parent[i];
@@ -330,7 +328,7 @@ VL_DEV StripRows ccl_load_rows(const uint32_t* mask, const CclGeom& g) {
 }
 
 // Rows of the tile into shared memory, strip unions, strip-run starts, their
-// counts before each word and per strip, and, with phi1, the seed columns:
+// counts before each word and per strip, and, with phi1, the seed columns (Smem::SEEDS):
 // all loads of a strip are in flight together.  Every warp then adds the
 // strips' counts up for itself: lane l returns the number of strip runs
 // before strip l (lane 31: all of them), the same in every warp.  s.base is
@@ -392,7 +390,7 @@ VL_DEV int ccl_tile_strips(Smem& s, StripRows rows, const uint32_t* phi1, const 
       if (lane == 0) { l0 = e0; l1 = e1; }
       if (lane == g.tww - 1) { q0 = e0; q1 = e1; }
       const uint32_t z = (a & (v0 | hdil(l0, c0, q0))) | (b & (v1 | hdil(l1, c1, q1)));
-      s.sd[k][lane] = first_in_segments(z, st);
+      if constexpr (Smem::SEEDS) s.sd[k][lane] = first_in_segments(z, st);
     }
   }
   __syncthreads();

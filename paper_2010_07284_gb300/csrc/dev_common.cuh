@@ -18,7 +18,6 @@ VL_DEV uint32_t vmask(int w, int W) {
 // Mask of bits 0..b inclusive.
 VL_DEV uint32_t le_mask(int b) { return b >= 31 ? 0xFFFFFFFFu : ((2u << b) - 1u); }
 
-// Loads that bypass L1: data written by other CTAs of the same launch.
 // Row and column of element i of a row-major grid of `cols` columns: a
 // 32-bit division while i < 2^32 (every word index, and every pixel index
 // of a grid under 2^32 pixels), else a 64-bit one.
@@ -33,6 +32,7 @@ VL_DEV void split_index(long long i, int cols, int& row, int& col) {
   }
 }
 
+// Loads that bypass L1: data written by other CTAs of the same launch.
 VL_DEV uint32_t ldcg(const uint32_t* p) { return __ldcg(p); }
 VL_DEV int32_t ldcg(const int32_t* p) { return __ldcg(p); }
 VL_DEV float ldcg(const float* p) { return __ldcg(p); }
@@ -102,18 +102,6 @@ VL_DEV uint32_t join_nibbles4(const uint32_t (&n)[4], int sub) {
   uint32_t w = second ? w1 : w0;
   w |= __shfl_xor_sync(0xFFFFFFFFu, second ? w0 : w1, 2);
   return w | __shfl_xor_sync(0xFFFFFFFFu, w, 1);
-}
-
-// Order-preserving map float -> uint32 (for selects on float keys); every
-// NaN maps to the largest key, after +infinity.
-VL_DEV uint32_t f2key(float f) {
-  if (f != f) return 0xFFFFFFFFu;
-  uint32_t u = __float_as_uint(f);
-  return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
-}
-VL_DEV float key2f(uint32_t k) {
-  uint32_t u = (k & 0x80000000u) ? (k & 0x7FFFFFFFu) : ~k;
-  return __uint_as_float(u);
 }
 
 // ---- number images: float or uint16 planes of H x pitch elements

@@ -39,9 +39,6 @@
 
 namespace vl {
 
-VL_DEV int sel_shift(int d) { return d == 0 ? 20 : d == 1 ? 8 : 0; }
-VL_DEV int sel_bins(int d) { return d == 2 ? 256 : SEL_BINS; }
-
 VL_DEV float sel_float(uint32_t key) { return __uint_as_float(sel_key_bits(key)); }
 
 constexpr int SEL_SAMPLE = 1024;
